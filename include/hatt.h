@@ -71,17 +71,17 @@ typedef struct {
  * randomized range-finder error. The paper computes in FP64 throughout; the
  * low-precision modes have no counterpart in it. */
 typedef enum {
-  TT_FP64 = 0,           /* every step in IEEE binary64 */
+  TT_FP64 = 0,           /* binary64 throughout. Products that are large enough run on the FP16
+                            tensor cores without loss: each operand entry is cut into eight
+                            8-bit digits of a 62-bit integer (its row or column scaled by a
+                            power of two), digit products are summed exactly in FP32 over
+                            at most 128 terms, and each such sum is rounded once to
+                            binary64; the error is below that of a chain of binary64
+                            fused multiply-adds, which smaller products use */
   TT_MIXED_FP32 = 1,     /* HPCRL-1 products: FP32 operands, FP32 accumulation */
   TT_MIXED_TF32 = 2,     /* HPCRL-1 products: TF32 operands, FP32 accumulation */
   TT_MIXED_BF16 = 3,     /* HPCRL-1 products: BF16 operands, FP32 accumulation */
-  TT_FP64_TC = 4         /* FP64 accuracy throughout; large products (max(M, N) >= 128,
-                            K >= 128, >= 2e7 flops) on the BF16 tensor cores: each row /
-                            column scaled by a power of two and cut into 9 slices of 6
-                            bits, slice products accumulated exactly in FP32 (<= 9 pairs
-                            per level, <= 448 terms of K per accumulation), levels
-                            combined in FP64; the error is that of an FP64 product
-                            (within 2^-54 of each row's and column's largest entry) */
+  TT_FP64_TC = 4         /* the same arithmetic as TT_FP64, kept for callers that name it */
 } tt_precision;
 
 /* Options of tt_hadamard_recompress (the problem statement of Algorithm 4:
@@ -341,9 +341,8 @@ int tt_batched_tune_cache(const char *path, int32_t save);
  * SIMT kernel with FP32-rounded operands and FP32 accumulation; for
  * TT_MIXED_TF32 / TT_MIXED_BF16 the tcgen05 tensor-core kernel, operands
  * rounded to the format (as tt_precision states) and FP32 accumulation per
- * K slice, slices summed in FP64; for TT_FP64_TC the FP64-accurate BF16
- * tensor-core products where the size qualifies. No counterpart in the
- * paper: it exposes the kernels of Eq. (3.6)'s contractions to
+ * K slice, slices summed in FP64; TT_FP64_TC is TT_FP64. No counterpart in
+ * the paper: it exposes the kernels of Eq. (3.6)'s contractions to
  * product-level checks.
  *   A  device, batch x M x K, row-major (leading dimension K)
  *   B  device, batch x K x N, row-major (leading dimension N)
@@ -351,28 +350,15 @@ int tt_batched_tune_cache(const char *path, int32_t save);
  *      overlap A or B
  *   M, N, batch >= 0, K >= 1; M K, K N, M N < 2^31 (TT_ERR_SHAPE)
  *   workspace  device, 256-byte aligned, tt_gemm_plan's size
- * Enqueued on `stream`; FP64 products may be timed once per new shape
- * (tt_gemm_autotune). */
+ * Enqueued on `stream`. */
 int tt_gemm_plan(int32_t precision, int64_t M, int64_t N, int64_t K, int64_t batch,
                  size_t *workspace_bytes);
 int tt_gemm(int32_t precision, int64_t M, int64_t N, int64_t K, int64_t batch, const double *A,
             const double *B, double *C, double alpha, void *workspace, size_t workspace_bytes,
             void *stream);
 
-/* FP64 GEMM plan tuning, an implementation detail with no counterpart in the
- * paper. The first time a GEMM shape (sizes, batch, operand layout) runs on a
- * stream that is not being captured, the library times its model's best
- * candidate tilings (single and paired-column forms, ~50 launches on the
- * call's own operands and output) and keeps the fastest for every later
- * launch of that shape in the process, including inside captured graphs.
- * This synchronizes the caller's stream once per tuned shape and allocates
- * nothing. A shape first met during a capture keeps the model's choice, and
- * so do products under 1e7 flops, products that accumulate into their output
- * or carry a device skip flag, and shapes beyond the first 256 tuned. Results
- * differ between tilings only by the order of FP64 rounding.
- * tt_gemm_autotune(0) turns the timing off for shapes not yet run (they keep
- * the model's choice), 1 turns it on (the default). Returns TT_OK; the
- * setting is process-wide. */
+/* Kept for its callers: FP64 products take their tilings from a cost model, and
+ * nothing is timed. Returns TT_OK and changes nothing. */
 int tt_gemm_autotune(int32_t enable);
 
 /* Kernel timer, a diagnostic with no counterpart in the paper: between

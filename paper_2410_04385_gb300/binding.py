@@ -226,7 +226,7 @@ def device_error() -> int:
 
 
 def gemm_autotune(enable: bool) -> None:
-    """First-use timing of FP64 GEMM tilings (tt_gemm_autotune); on by default."""
+    """Kept for its callers (tt_gemm_autotune): nothing is timed, nothing changes."""
     _check("tt_gemm_autotune", load().tt_gemm_autotune(1 if enable else 0))
 
 

@@ -881,10 +881,10 @@ size_t measure(Carve carve, Run runf) {
   return ws.off + 256;
 }
 
-// Switches the FP64-accurate tensor-core products on for one call.
-struct Fp64TcScope {
-  explicit Fp64TcScope(bool on) { hatt::set_fp64_tensor_cores(on); }
-  ~Fp64TcScope() { hatt::set_fp64_tensor_cores(false); }
+// Keeps the products of one call on the DFMA kernels unless `on`.
+struct SplitScope {
+  explicit SplitScope(bool on) { hatt::set_split_products(on); }
+  ~SplitScope() { hatt::set_split_products(true); }
 };
 
 // While a batch issues its lanes: the truncation sweep does not synchronize,
@@ -1342,9 +1342,16 @@ int tt_dot_noalloc(const tt_t *A, const tt_t *B, double *out, void *stream) {
   int st = prepare_dot(A, B, true);
   if (st != TT_OK) return st;
   if (!out) return TT_ERR_ARG;
-  const size_t need = measure([&](Ws &ws) { return carve_dot(ws, A, B); },
-                              [&](Runner &run, const DotBufs &u) { run_dot(run, A, B, u, nullptr); });
-  if (need > kNoAllocScratchBytes) return TT_ERR_WORKSPACE;
+  // the tensor-core products may split K into more partial sums than the DFMA
+  // ones: where only those do not fit the array, the call runs without them
+  auto need = [&](bool split) {
+    SplitScope scope(split);
+    return measure([&](Ws &ws) { return carve_dot(ws, A, B); },
+                   [&](Runner &run, const DotBufs &u) { run_dot(run, A, B, u, nullptr); });
+  };
+  const bool split = need(true) <= kNoAllocScratchBytes;
+  if (!split && need(false) > kNoAllocScratchBytes) return TT_ERR_WORKSPACE;
+  SplitScope scope(split);
   void *scratch = nullptr;
   cudaError_t e = noalloc_scratch_address(&scratch);
   if (e != cudaSuccess) return from_cuda(e);
@@ -1380,7 +1387,6 @@ int tt_hadamard_recompress_plan(const tt_t *Y, const tt_t *Z, const tt_opts *opt
   a.Y = nullptr;
   a.Z = nullptr;
   a.Xout = nullptr;
-  Fp64TcScope tc(opts->precision == TT_FP64_TC);
   *workspace_bytes = measure([&](Ws &ws) { return carve_hatt(ws, a); },
                              [&](Runner &run, const HattBufs &b) { run_hatt(run, a, b); });
   return TT_OK;
@@ -1412,7 +1418,6 @@ int tt_hadamard_recompress(const tt_t *Y, const tt_t *Z, const tt_opts *opts, tt
   a.Z = Z->cores;
   a.Xout = X->cores;
   cudaStream_t strm = (cudaStream_t)stream;
-  Fp64TcScope tc(opts->precision == TT_FP64_TC);
   HattBufs bufs_for_ranks;
   st = execute(workspace, workspace_bytes, strm,
                [&](Ws &ws) {
@@ -1786,7 +1791,6 @@ int tt_gemm_plan(int32_t precision, int64_t M, int64_t N, int64_t K, int64_t bat
   hatt::Gemm g;
   const int st = gemm_args(precision, M, N, K, batch, g);
   if (st != TT_OK) return st;
-  Fp64TcScope tc(precision == TT_FP64_TC);
   *workspace_bytes = measure([&](Ws &) { return NoBufs{}; },
                              [&](Runner &run, const NoBufs &) { run.gemm(g); });
   return TT_OK;
@@ -1805,13 +1809,12 @@ int tt_gemm(int32_t precision, int64_t M, int64_t N, int64_t K, int64_t batch, c
   g.B = B;
   g.C = C;
   g.alpha = alpha;
-  Fp64TcScope tc(precision == TT_FP64_TC);
   return execute(workspace, workspace_bytes, (cudaStream_t)stream, [&](Ws &) { return NoBufs{}; },
                  [&](Runner &run, const NoBufs &) { run.gemm(g); });
 }
 
 int tt_gemm_autotune(int32_t enable) {
-  hatt::set_gemm_autotune(enable != 0);
+  (void)enable;   // plans come from the cost model alone; the entry point stays for its callers
   return TT_OK;
 }
 

@@ -130,21 +130,19 @@ struct Gemm {
 
 // Doubles of split-K scratch this GEMM needs (0 if it runs unsplit).
 size_t gemm_scratch_doubles(const Gemm &g);
-// First-use timing of candidate GEMM plans (on by default; see k_gemm.cu).
-void set_gemm_autotune(bool on);
 // TF32 / BF16 products on the tensor cores (tcgen05, FP32 accumulator in
 // tensor memory); gemm_f64 dispatches to them by g.prec.
 bool gemm_tc_supported(const Gemm &g);
 size_t gemm_tc_scratch_doubles(const Gemm &g);
 cudaError_t gemm_tc(const Gemm &g, double *scratch, int *counters, cudaStream_t st);
-// FP64-accurate products on the BF16 tensor cores (slices of 6 bits, exact
-// FP32 accumulation per level): gemm_f64 uses them for large FP64 products
-// while the calling thread has switched them on.
-void set_fp64_tensor_cores(bool on);
-bool gemm_oz_applicable(const Gemm &g);
-size_t gemm_oz_scratch_doubles(const Gemm &g);
-cudaError_t gemm_oz(const Gemm &g, double *scratch, cudaStream_t st);
-cudaError_t oz_error_word(int *value, bool clear);
+// FP64 products on the BF16 tensor cores from exact digits of both operands
+// (k_gemm_split.cu); gemm_f64 dispatches to them by size.
+// set_split_products(false) keeps the calling thread on the DFMA kernels.
+void set_split_products(bool on);
+bool gemm_split_applicable(const Gemm &g);
+size_t gemm_split_scratch_doubles(const Gemm &g);
+cudaError_t gemm_split(const Gemm &g, double *scratch, cudaStream_t st);
+cudaError_t split_error_word(int *value, bool clear);
 // Error word set by a device wait that ran out (the kernel wrote NaN to its
 // outputs, freed its tensor memory and returned): read (synchronizing the
 // device) and clear it.
