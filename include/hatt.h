@@ -279,13 +279,16 @@ int tt_philox4x32_10(const uint32_t *ctr, uint32_t key0, uint32_t key1, uint32_t
 int64_t tt_launch_count(void);
 
 /* ---------------------------------------------------------------- batched
- * Many independent recompressions in ONE persistent launch. Each pair runs
- * HaTT-1 (Algorithm 3, then Algorithm 4) exactly as tt_hadamard_recompress
+ * Many independent recompressions in one call: the small pairs in ONE
+ * persistent launch of the task engine, pairs whose contractions have 10 MFLOP
+ * or more, where the plan predicts a gain, as launch sequences on up to 16
+ * streams that the plan owns (their products run on the tensor cores). Each pair
+ * runs HaTT-1 (Algorithm 3, then Algorithm 4) exactly as tt_hadamard_recompress
  * does, with the sketch rank as output rank (no truncation sweep). The paper
  * recompresses one product at a time; the task engine has no counterpart in
- * it. Every pair's launch sequence becomes a chain of stages (its GEMMs, the
+ * it. In the engine a pair's launch sequence becomes a chain of stages (its GEMMs, the
  * Cholesky QR passes, norms, sketch cores) split into tasks (output tiles,
- * row blocks, element chunks). One queue holds the tasks of all pairs,
+ * row blocks, element chunks). One queue holds the tasks of all its pairs,
  * interleaved so that the pairs with the longest chains (most stages) start
  * first and, within a round of stages, the pairs with the most predicted
  * flops go first. Resident CTAs take tasks in queue order; a task waits, by a
@@ -306,15 +309,18 @@ int64_t tt_launch_count(void);
  *   reported), and with autotune = 1 times the candidate tile shapes of the
  *   48 GEMM shape buckets with the most flops that are not yet in the
  *   process-wide cache (the others keep an analytic choice); uploads the task
- *   tables. Synchronizes `stream`; not allowed while it is being captured.
+ *   tables and creates the plan's streams on the current device. Synchronizes
+ *   `stream`; not allowed while it is being captured.
  * run: clears the control words and enqueues the persistent launch on
- *   `stream` (no synchronization; capturable once bound). spin_cap bounds each
+ *   `stream` and the larger pairs on the plan's streams, forked from and joined
+ *   to `stream` (no synchronization; capturable once bound). spin_cap bounds each
  *   wait (polls of ~0.25 us; once any wait has run out every later wait gives
  *   up at once and the results are invalid).
  * status: reads the status word of the last run (synchronizes `stream`):
  *   TT_OK, TT_ERR_TIMEOUT if a wait ran out, TT_ERR_NONFINITE if a norm or a
  *   Gram matrix was not finite (NaN or Inf in an input), TT_ERR_BREAKDOWN.
- * info: number of stages and tasks of the bound plan and resident CTAs.
+ * info: number of stages and tasks of the bound plan's engine launch (0 when
+ *   every pair runs on a stream) and its resident CTAs.
  * profile: sums over the CTAs of the last run's profile words into out (host
  *   int64[24]): [0] cycles from each CTA's start to its end, [1] cycles
  *   polling for prerequisites, [2] cycles taking tickets, [8 + t] cycles

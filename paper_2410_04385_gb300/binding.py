@@ -611,9 +611,10 @@ def device_status() -> int:
 
 
 class BatchedRecompressor:
-    """Many independent pairs recompressed by ONE persistent launch of the task
-    engine (tt_batched_*). Plans once, owns every output buffer and the
-    workspace; `run` enqueues the launch (capturable after construction)."""
+    """Many independent pairs recompressed in one call (tt_batched_*): the small
+    ones by one persistent launch of the task engine, the larger ones on streams
+    that the plan owns. Plans once, owns every output buffer and the workspace;
+    `run` enqueues the work (capturable after construction)."""
 
     def __init__(self, pairs, autotune: bool = True, stream=None):
         """pairs: list of (Y cores, Z cores, options dict) with CUDA float64

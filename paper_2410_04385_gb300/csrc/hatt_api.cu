@@ -10,6 +10,8 @@
 #include <atomic>
 #include <cmath>
 #include <cstdio>
+#include <cstdlib>
+#include <cstring>
 #include <map>
 #include <memory>
 #include <mutex>
@@ -888,13 +890,16 @@ struct SplitScope {
 };
 
 // While a batch issues its lanes: the truncation sweep does not synchronize,
-// and kernels are launched without programmatic serialization.
+// kernels are launched without programmatic serialization, and health bits go
+// to `status` (nullptr: the device error word).
 struct BatchScope {
-  BatchScope() {
+  explicit BatchScope(int *status = nullptr) {
     hatt::set_host_sync(false);
     hatt::set_programmatic_launch(false);
+    hatt::set_health_word(status);
   }
   ~BatchScope() {
+    hatt::set_health_word(nullptr);
     hatt::set_host_sync(true);
     hatt::set_programmatic_launch(true);
   }
@@ -942,6 +947,7 @@ struct EnginePair {
   HattArgs a;
   size_t ws_off = 0, ws_bytes = 0;   // the pair's region of the workspace
   double cost = 0.0;                 // predicted flops (Section 4 model)
+  int lane = -1;                     // >= 0: runs on that stream of the plan, not in the engine
   std::vector<hatt::EngineStage> stages;
   std::vector<int> group;            // stages with the same group id share prerequisites
 };
@@ -1134,10 +1140,100 @@ double eng_stage_flops(const hatt::EngineStage &s) {
   }
 }
 
+// Which pairs leave the task engine for a stream of their own. The engine's tasks
+// are DFMA tiles and one-block factorizations, and a pair's stages follow each
+// other: its time is the longest chain (per core ~150 us, 40 us per column of the
+// QR and the QR's Gram matrix on one SM) plus the batch's products at ~0.9
+// TFLOP/s. On a stream a pair's products run on the tensor cores, and its
+// launches cost the issuing thread ~57 us per core, one pair after the other. The
+// plan takes the split of the pairs (longest chains to the streams) with the
+// least sum of both. Pairs under kLaneFlops stay in the engine.
+// Measured (ms, all in the engine and all on streams): 12 pairs of 7 to 18 GFLOP
+// 451 and 56, 8 of 0.5 to 1.4 GFLOP 65 and 6.9, 8 of 60 to 170 MFLOP 17 and 3.6, 12
+// of 30 to 50 MFLOP 10 and 4.0, 48 of 25 to 60 MFLOP 12.8 and 15.9, 24 of 1 to 10
+// MFLOP 6.6 and 4.9, 24 under 4 MFLOP 3.2 and 4.1.
+constexpr double kLaneFlops = 1e7;
+constexpr int kBatchLanes = 16;
+
+struct PairCost {
+  double flops = 0.0;                // contractions of Section 4
+  double chain_us = 0.0;             // in the engine
+  double issue_us = 0.0;             // on a stream
+};
+
+PairCost pair_cost(const HattArgs &a) {
+  PairCost p;
+  for (int k = 0; k < a.d; ++k) {
+    const double n = (double)a.n[k], r0 = (double)a.r[k], r1 = (double)a.r[k + 1], s0 = (double)a.s[k],
+                 s1 = (double)a.s[k + 1], l0 = (double)a.ell[k], l1 = (double)a.ell[k + 1];
+    if (k > 0) p.flops += 2.0 * n * (r1 * s1 * l0 * l1 + r1 * s0 * s1 * l0 + r0 * r1 * s0 * l0 +
+                                     l0 * r0 * s0 * s1 + l0 * r0 * r1 * s1);
+    if (k + 1 == a.d) break;
+    p.flops += 4.0 * l0 * n * l1 * r1 * s1;
+    p.chain_us += 150.0 + 40.0 * l1 + l0 * n * l1 * l1 / 1650.0;
+    p.issue_us += 57.0;
+  }
+  return p;
+}
+
+// HATT_BATCH_FORM=engine / lanes (read once): a test hook that sends every pair
+// one way.
+int batch_form() {
+  static const int form = [] {
+    const char *v = getenv("HATT_BATCH_FORM");
+    return v == nullptr ? 0 : strcmp(v, "engine") == 0 ? 1 : strcmp(v, "lanes") == 0 ? 2 : 0;
+  }();
+  return form;
+}
+
+// Pairs that run on streams, the most expensive first.
+std::vector<int> lane_pairs(const std::vector<PairCost> &cost) {
+  std::vector<int> order;
+  double flops = 0.0, rest_chain = 0.0;            // of the pairs that stay
+  for (int j = 0; j < (int)cost.size(); ++j) {
+    flops += cost[j].flops;
+    if (batch_form() == 2 || (batch_form() == 0 && cost[j].flops >= kLaneFlops)) order.push_back(j);
+    else rest_chain = std::max(rest_chain, cost[j].chain_us);
+  }
+  std::stable_sort(order.begin(), order.end(),
+                   [&](int x, int y) { return cost[x].chain_us > cost[y].chain_us; });
+  size_t take = batch_form() == 2 ? order.size() : 0;
+  double best = 1e300, issue = 0.0;
+  for (size_t k = 0; k <= order.size() && batch_form() == 0; ++k) {
+    // the k longest chains on streams, the others in the engine
+    const double chain = std::max(rest_chain, k < order.size() ? cost[order[k]].chain_us : 0.0);
+    const double t = issue + (chain > 0.0 ? chain + flops / 0.9e6 : 0.0);
+    if (t < best) {
+      best = t;
+      take = k;
+    }
+    if (k < order.size()) {
+      issue += cost[order[k]].issue_us;
+      flops -= cost[order[k]].flops;
+    }
+  }
+  order.resize(take);
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cost[x].flops > cost[y].flops; });
+  return order;
+}
+
 }  // namespace
 
-// The plan behind tt_batched_* (opaque to callers).
+// The plan behind tt_batched_* (opaque to callers). It owns the streams and
+// events of its larger pairs, so that plans never share any: two of them may run
+// from two threads, one of them under capture.
 struct tt_batch_plan {
+  ~tt_batch_plan() {
+    for (cudaStream_t s : lane_streams) cudaStreamDestroy(s);
+    for (cudaEvent_t e : lane_done) cudaEventDestroy(e);
+    if (fork) cudaEventDestroy(fork);
+  }
+  std::vector<cudaStream_t> lane_streams;
+  std::vector<cudaEvent_t> lane_done;
+  cudaEvent_t fork = nullptr;
+  int lanes = 0;
+  std::vector<int> lane_order;       // the streams' pairs, the most expensive first
+
   int count = 0;
   std::vector<EnginePair> pairs;
   size_t ws_bytes = 0;
@@ -1888,6 +1984,7 @@ int tt_batched_plan_create(int32_t count, const tt_t *Y, const tt_t *Z, const tt
   P->pairs.resize(count);
   size_t off = 0;
   long long flag_ints = 0;
+  std::vector<PairCost> cost(count);
   for (int j = 0; j < count; ++j) {
     EnginePair &ep = P->pairs[j];
     int st = prepare_hatt(&Y[j], &Z[j], &opts[j], true, ep.a);
@@ -1903,11 +2000,31 @@ int tt_batched_plan_create(int32_t count, const tt_t *Y, const tt_t *Z, const tt
     ep.a.Z = Z[j].cores;
     ep.a.Xout = X[j].cores;
     for (int k = 0; k <= ep.a.d; ++k) X[j].r[k] = ep.a.outb[k];
+    cost[j] = pair_cost(ep.a);
+  }
+  {   // streams: the most expensive pair first, each to the least loaded one (LPT)
+    P->lane_order = lane_pairs(cost);
+    P->lanes = std::min<int>((int)P->lane_order.size(), kBatchLanes);
+    std::vector<double> load(std::max(P->lanes, 1), 0.0);
+    for (int j : P->lane_order) {
+      const int l = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+      P->pairs[j].lane = l;
+      load[l] += cost[j].flops;
+    }
+  }
+  for (int j = 0; j < count; ++j) {
+    EnginePair &ep = P->pairs[j];
     ep.ws_off = off;
-    ep.ws_bytes = eng_pair_bytes(ep.a);
+    if (ep.lane >= 0) {
+      ep.ws_bytes = (measure([&](Ws &ws) { return carve_hatt(ws, ep.a); },
+                             [&](Runner &run, const HattBufs &b) { run_hatt(run, ep.a, b); }) + 255) &
+                    ~(size_t)255;
+    } else {
+      ep.ws_bytes = eng_pair_bytes(ep.a);
+      for (int k = 0; k <= ep.a.d; ++k) P->max_c = std::max<int>(P->max_c, (int)ep.a.ell[k]);
+    }
     off += ep.ws_bytes;
     flag_ints += 4LL * ep.a.d;
-    for (int k = 0; k <= ep.a.d; ++k) P->max_c = std::max<int>(P->max_c, (int)ep.a.ell[k]);
   }
   // control words: head, status, per-pair completion counters, QR flags, then
   // the per-CTA profile words (all cleared every run)
@@ -1923,6 +2040,7 @@ int tt_batched_plan_create(int32_t count, const tt_t *Y, const tt_t *Z, const tt
   int *fq = reinterpret_cast<int *>(fake + ctl_off) + 2 + count;
   for (int j = 0; j < count; ++j) {
     EnginePair &ep = P->pairs[j];
+    if (ep.lane >= 0) continue;
     int st = eng_record_pair(ep, fake + ep.ws_off, fq, j, ops);
     if (st != TT_OK) return st;
     fq += 4 * ep.a.d;
@@ -1971,11 +2089,24 @@ int tt_batched_plan_bind(tt_batch_plan *P, void *workspace, size_t workspace_byt
   int *fq = P->qflags_all;
   for (int j = 0; j < P->count; ++j) {
     EnginePair &ep = P->pairs[j];
+    if (ep.lane >= 0) continue;
     int s = eng_record_pair(ep, ws + ep.ws_off, fq, j, ops);
     if (s != TT_OK) return s;
     fq += 4 * ep.a.d;
   }
   cudaError_t e = cudaMemsetAsync(ctl, 0, P->flags_bytes, st);
+  if (e == cudaSuccess && P->lanes > 0 && !P->fork)
+    e = cudaEventCreateWithFlags(&P->fork, cudaEventDisableTiming);
+  while (e == cudaSuccess && (int)P->lane_streams.size() < P->lanes) {
+    cudaStream_t s = nullptr;
+    e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+    if (e == cudaSuccess) P->lane_streams.push_back(s);
+  }
+  while (e == cudaSuccess && (int)P->lane_done.size() < P->lanes) {
+    cudaEvent_t v = nullptr;
+    e = cudaEventCreateWithFlags(&v, cudaEventDisableTiming);
+    if (e == cudaSuccess) P->lane_done.push_back(v);
+  }
   if (e != cudaSuccess) return from_cuda(e);
   if (autotune) {
     int tuned = 0;
@@ -1986,8 +2117,9 @@ int tt_batched_plan_bind(tt_batch_plan *P, void *workspace, size_t workspace_byt
   const size_t sb = P->stages.size() * sizeof(hatt::EngineStage);
   const size_t tb = P->tasks.size() * sizeof(hatt::EngineTask);
   if (P->tables_off + sb + tb > P->ws_bytes) return TT_ERR_WORKSPACE;
-  e = cudaMemcpyAsync(ws + P->tables_off, P->stages.data(), sb, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess)
+  if (sb > 0)
+    e = cudaMemcpyAsync(ws + P->tables_off, P->stages.data(), sb, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess && tb > 0)
     e = cudaMemcpyAsync(ws + P->tables_off + sb, P->tasks.data(), tb, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = hatt::engine_blocks(P->max_c, &P->blocks);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);             // host tables may change later
@@ -2002,9 +2134,40 @@ int tt_batched_run(tt_batch_plan *P, int64_t spin_cap, void *stream) {
   const auto *stages = reinterpret_cast<const hatt::EngineStage *>(P->ws + P->tables_off);
   const auto *tasks = reinterpret_cast<const hatt::EngineTask *>(
       P->ws + P->tables_off + P->stages.size() * sizeof(hatt::EngineStage));
-  e = hatt::engine_launch(stages, tasks, (int)P->tasks.size(), P->head, P->done, P->status,
-                          (long long)spin_cap, P->max_c, P->blocks, P->prof, st);
-  return from_cuda(e);
+  // the larger pairs, each on its stream of the plan, forked from the caller's
+  int first_error = TT_OK;
+  if (P->lanes > 0) {
+    e = cudaEventRecord(P->fork, st);
+    for (int l = 0; l < P->lanes && e == cudaSuccess; ++l)
+      e = cudaStreamWaitEvent(P->lane_streams[l], P->fork, 0);
+    if (e != cudaSuccess) return from_cuda(e);
+  }
+  if (!P->tasks.empty()) {
+    e = hatt::engine_launch(stages, tasks, (int)P->tasks.size(), P->head, P->done, P->status,
+                            (long long)spin_cap, P->max_c, P->blocks, P->prof, st);
+    first_error = from_cuda(e);
+  }
+  {
+    static_assert(hatt::kHealthTimeout == hatt::kEngineTimeout &&
+                      hatt::kHealthNonfinite == hatt::kEngineNonfinite &&
+                      hatt::kHealthBreakdown == hatt::kEngineBreakdown,
+                  "both forms of a pair set the same status bits");
+    BatchScope scope(P->status);
+    for (int j : P->lane_order) {
+      if (first_error != TT_OK) break;
+      const EnginePair &ep = P->pairs[j];
+      first_error = execute(P->ws + ep.ws_off, ep.ws_bytes, P->lane_streams[ep.lane],
+                            [&](Ws &ws) { return carve_hatt(ws, ep.a); },
+                            [&](Runner &run, const HattBufs &b) { run_hatt(run, ep.a, b); });
+    }
+  }
+  // every stream that was forked joins, also after an error
+  for (int l = 0; l < P->lanes; ++l) {
+    e = cudaEventRecord(P->lane_done[l], P->lane_streams[l]);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, P->lane_done[l], 0);
+    if (e != cudaSuccess && first_error == TT_OK) first_error = from_cuda(e);
+  }
+  return first_error;
 }
 
 int tt_batched_status(tt_batch_plan *P, void *stream, int32_t *status) {

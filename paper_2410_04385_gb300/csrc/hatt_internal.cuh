@@ -154,6 +154,11 @@ cudaError_t clear_device_error();
 // bit owns its word; read_device_error ORs them.
 constexpr int kHealthTimeout = 1, kHealthNonfinite = 2, kHealthBreakdown = 4;
 cudaError_t qr_health_word(int *value, bool clear);
+// Where the calling thread's next factorizations and norms note their bits: a
+// device word of the caller (a batched plan's status), or nullptr for the
+// device error word.
+void set_health_word(int *word);
+int *health_target();
 cudaError_t misc_health_word(int *value, bool clear);
 // Enqueue; `scratch` must hold gemm_scratch_doubles(g) doubles.
 cudaError_t gemm_f64(const Gemm &g, double *scratch, cudaStream_t st);

@@ -94,7 +94,7 @@ __global__ void philox_raw_kernel(const uint32_t *ctr, uint32_t k0, uint32_t k1,
 
 __global__ void __launch_bounds__(kThreads)
 inv_norm_kernel(const double *x, long long count, double *out, double *partials,
-                unsigned int *ticket) {
+                unsigned int *ticket, int *health) {
   pdl_enter();
   __shared__ double red[kThreads];
   __shared__ bool last;
@@ -126,7 +126,7 @@ inv_norm_kernel(const double *x, long long count, double *out, double *partials,
   }
   if (threadIdx.x == 0) {
     const double ss = red[0];
-    if (!isfinite(ss)) atomicOr(&g_misc_health, kHealthNonfinite);
+    if (!isfinite(ss)) atomicOr(health != nullptr ? health : &g_misc_health, kHealthNonfinite);
     out[0] = ss > 0.0 ? 1.0 / sqrt(ss) : 1.0;
     *ticket = 0u;
   }
@@ -230,10 +230,16 @@ cudaError_t philox_raw(const uint32_t *ctr, uint32_t k0, uint32_t k1, uint32_t *
   return cudaGetLastError();
 }
 
+namespace {
+thread_local int *t_health_word = nullptr;
+}
+void set_health_word(int *word) { t_health_word = word; }
+int *health_target() { return t_health_word; }
+
 cudaError_t inv_norm(const double *x, long long count, double *out, double *partials,
                      unsigned int *ticket, cudaStream_t st) {
   const int blocks = (int)std::max<long long>(1, std::min<long long>((count + kThreads - 1) / kThreads, 2 * 152));
-  launch_k(inv_norm_kernel, blocks, kThreads, 0, st, x, count, out, partials, ticket);
+  launch_k(inv_norm_kernel, blocks, kThreads, 0, st, x, count, out, partials, ticket, health_target());
   note_launch();
   return cudaGetLastError();
 }

@@ -47,6 +47,8 @@ namespace hatt {
 namespace {
 
 __device__ int g_qr_health = 0;   // kHealthNonfinite / kHealthBreakdown bits
+// The word a factorization notes them in: the caller's (set_health_word) or ours.
+__device__ __forceinline__ int *health_word(int *word) { return word != nullptr ? word : &g_qr_health; }
 
 constexpr int kPasses = 6;
 constexpr int kCholThreads = 256;
@@ -123,7 +125,8 @@ __device__ __forceinline__ void warp_stats(long long &dev, long long &dmax, doub
 // (the value a failed pivot takes) are scaled alike.
 __device__ __forceinline__ void chol_pivot(double *G, int ld, int j, const unsigned char *zero_col,
                                            double floor_piv, double clamp, int attempt,
-                                           double *rinv2, double *pivots, unsigned char *fail) {
+                                           double *rinv2, double *pivots, unsigned char *fail,
+                                           int *health) {
   if (zero_col[j]) {
     rinv2[j] = 1.0;
     pivots[j] = 1.0;
@@ -132,7 +135,7 @@ __device__ __forceinline__ void chol_pivot(double *G, int ld, int j, const unsig
   double piv = G[j * ld + j];
   if (!(piv > floor_piv)) {
     if (attempt == 0) fail[j] = 1;
-    else atomicOr(&g_qr_health, kHealthBreakdown);
+    else atomicOr(health_word(health), kHealthBreakdown);
     piv = clamp;
   }
   pivots[j] = piv;
@@ -159,7 +162,7 @@ __device__ __forceinline__ void chol_pivot(double *G, int ld, int j, const unsig
 // publication scales row j by y_j^2. G is read through L2 (__ldcg): in the
 // fused form other blocks of the same launch wrote it.
 __device__ __forceinline__ void chol_factor(const double *Gg, double *Ut_g, double *y_g, int c,
-                                            int m, int *flags, double *sm) {
+                                            int m, int *flags, int *health, double *sm) {
   const int ld = c + 1;
   double *G = sm;                                   // c x ld, upper triangle is updated
   __shared__ double s_red[3][kCholThreads / 32];
@@ -225,7 +228,7 @@ __device__ __forceinline__ void chol_factor(const double *Gg, double *Ut_g, doub
   // it, leave S as it is and stop this QR (every later pass is a no-op)
   if (__syncthreads_or(bad)) {
     if (tid == 0) {
-      atomicOr(&g_qr_health, kHealthNonfinite);
+      atomicOr(health_word(health), kHealthNonfinite);
       flags[0] = 1;
       flags[1] = 1;
     }
@@ -284,7 +287,7 @@ __device__ __forceinline__ void chol_factor(const double *Gg, double *Ut_g, doub
     __syncthreads();
     const double floor_piv = (attempt == 0) ? (double)c * u * s_diag_max * sc : 0.0;
     const double clamp = fmax(shift, 1e-300) * sc;
-    if (tid == 0) chol_pivot(G, ld, 0, s_zero, floor_piv, clamp, attempt, s_rinv2, s_piv, s_failc);
+    if (tid == 0) chol_pivot(G, ld, 0, s_zero, floor_piv, clamp, attempt, s_rinv2, s_piv, s_failc, health);
     __syncthreads();
     bool failed = false;
     for (int j = 0; j < c; ++j) {
@@ -299,7 +302,7 @@ __device__ __forceinline__ void chol_factor(const double *Gg, double *Ut_g, doub
         const double rji = rowj[i] * y2;
         for (int l = i + lane; l < c; l += 32) G[i * ld + l] = fma(-rji, rowj[l], G[i * ld + l]);
         __syncwarp();
-        if (lane == 0) chol_pivot(G, ld, i, s_zero, floor_piv, clamp, attempt, s_rinv2, s_piv, s_failc);
+        if (lane == 0) chol_pivot(G, ld, i, s_zero, floor_piv, clamp, attempt, s_rinv2, s_piv, s_failc, health);
       }
       // trailing update of the rows below by warps 1..7 on a 14 x 16 grid:
       // warp 0 carries the pivot chain and takes no share of it
@@ -346,14 +349,14 @@ __device__ __forceinline__ void chol_factor(const double *Gg, double *Ut_g, doub
 }
 
 __global__ void __launch_bounds__(kCholThreads)
-chol_inv_kernel(const double *Gg, double *Ut_g, double *y_g, int c, int m, int *flags) {
+chol_inv_kernel(const double *Gg, double *Ut_g, double *y_g, int c, int m, int *flags, int *health) {
   pdl_enter();
   if (flags[0]) {
     if (threadIdx.x == 0) flags[1] = 1;
     return;
   }
   extern __shared__ double sm[];
-  chol_factor(Gg, Ut_g, y_g, c, m, flags, sm);
+  chol_factor(Gg, Ut_g, y_g, c, m, flags, health, sm);
 }
 
 // Q = S R^{-1} = (S U~^{-1}) D^{-1}, one warp per row, in place. The unit
@@ -639,7 +642,7 @@ qr_fused_kernel(double *S, int m, int c, long long ldS, double *G, double *Ut, d
     if (!grid_barrier(bar, epoch, spin_cap)) return;
     for (int t = bid * kWarps + warp; t < T; t += nb * kWarps) gram_entry(part, nb, c, t, G);
     if (!grid_barrier(bar, epoch, spin_cap)) return;
-    if (bid == 0) chol_factor(G, Ut, y, c, m, flags, sm);
+    if (bid == 0) chol_factor(G, Ut, y, c, m, flags, nullptr, sm);
     if (!grid_barrier(bar, epoch, spin_cap)) return;
     const int done = __ldcg(flags), skip = __ldcg(flags + 1);
     if (skip) return;                      // orthonormal already (or a non-finite G)
@@ -778,7 +781,7 @@ cudaError_t qr_inplace(double *S, int m, int c, long long ldS, double *scratch, 
     note_launch();
     launch_k(gram_sum_kernel, sum_blocks, kCholThreads, 0, st, part, nb, c, G, flags);
     note_launch();
-    launch_k(chol_inv_kernel, 1, kCholThreads, chol_smem(c), st, G, Ut, y, c, m, flags);
+    launch_k(chol_inv_kernel, 1, kCholThreads, chol_smem(c), st, G, Ut, y, c, m, flags, health_target());
     note_launch();
     launch_k(trsm_rows_kernel, blocks, kTrsmThreads, trsm_smem(c), st, S, m, c, ldS, Ut, y, flags);
     note_launch();
