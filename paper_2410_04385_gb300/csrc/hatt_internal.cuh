@@ -239,9 +239,6 @@ constexpr int kMaxDevices = 64;
 cudaError_t refine_cluster_available(bool *ok);
 cudaError_t refine_cluster(const double *G, int c, double *U, double floor_norm, const int *skip,
                            cudaStream_t st);
-// FP32 eigenvectors of the symmetric c x c matrix G (columns of U, decreasing
-// eigenvalues), the refinement's start (k_eig.cu); *skip != 0 leaves U untouched.
-cudaError_t eig_start(const double *G, int c, double *U, const int *skip, cudaStream_t st);
 // Eigenvectors (columns of U, c x c row-major) of the symmetric c x c matrix G.
 size_t sym_eig_scratch_doubles(int c);
 cudaError_t sym_eig(const double *G, int c, double *U, double *scratch, cudaStream_t st);

@@ -990,25 +990,15 @@ size_t trunc_scratch_doubles(int la, int n, int lb, int lm, int nm) {
 // state[j] != 0 turns step j into no-ops (state[0] also the FP32 start): the
 // caller clears state[0..kEigSteps) or sets it to skip everything, and a step
 // whose correction is below kConverged sets the flags of all later steps.
-// ordered: the start of tolerance mode. Its spectra reach below what FP32
-// resolves, where the refinement keeps whatever basis the start gives an
-// unresolved group, so results there depend on the order of the start's sums
-// (a 24-of-34 cut of u * u moves by 1e-3); eig_tridiag32_kernel keeps that
-// order. A rank cut alone (and HPCRL-2's selection) takes eig_start: 58 us
-// against 116 at c = 50, 124 against 400 at c = 90, same results to rounding.
 static cudaError_t eigvecs(const double *A, int c, double *Ua, double *Ub, double floor_norm,
-                           int *state, bool ordered, const Layout &L, cudaStream_t st) {
+                           int *state, const Layout &L, cudaStream_t st) {
   cudaError_t e;
 #define HATT_TRY(x) do { e = (x); if (e != cudaSuccess) return e; } while (0)
-  if (ordered) {
-    HATT_TRY(cudaFuncSetAttribute(eig_tridiag32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)eig_smem(kMaxSmall)));
-    launch_k(eig_tridiag32_kernel, 1, kEigThreads, eig_smem(c), st, A, c, Ua, state);
-    note_launch();
-    HATT_TRY(cudaGetLastError());
-  } else {
-    HATT_TRY(eig_start(A, c, Ua, state, st));
-  }
+  HATT_TRY(cudaFuncSetAttribute(eig_tridiag32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)eig_smem(kMaxSmall)));
+  launch_k(eig_tridiag32_kernel, 1, kEigThreads, eig_smem(c), st, A, c, Ua, state);
+  note_launch();
+  HATT_TRY(cudaGetLastError());
   if (c <= kEigFusedMax) {          // all refinement steps in one cluster launch
     bool ok = false;
     HATT_TRY(refine_cluster_available(&ok));
@@ -1057,7 +1047,7 @@ cudaError_t trunc_step(double *Xk, int la, int n, int lb, double *Xkm1, int lm, 
   int *state1 = L.flags + 8, *state2 = L.flags + 16;
   HATT_TRY(gemm_f64(g_gram(Xk, la, N, L.G), L.gs, st));
   HATT_TRY(cudaMemsetAsync(state1, 0, kEigSteps * sizeof(int), st));
-  HATT_TRY(eigvecs(L.G, la, L.U0, L.U1, 0.0, state1, deep, L, st));
+  HATT_TRY(eigvecs(L.G, la, L.U0, L.U1, 0.0, state1, L, st));
   double *U = L.U0;
   HATT_TRY(gemm_f64(g_tn(U, Xk, la, N, N, L.B1, N), L.gs, st));
   if (deep) {
@@ -1080,7 +1070,7 @@ cudaError_t trunc_step(double *Xk, int la, int n, int lb, double *Xkm1, int lm, 
         HATT_TRY(cudaStreamSynchronize(st));
         if (skip) break;
       }
-      HATT_TRY(eigvecs(L.H, la, L.V0, L.V1, 1.0, state2, true, L, st));
+      HATT_TRY(eigvecs(L.H, la, L.V0, L.V1, 1.0, state2, L, st));
       HATT_TRY(gemm_f64(g_nn(Ua, L.V0, la, la, la, Ub), L.gs, st));              // Ub = Ua V
       g = g_tn(Ub, Xk, la, N, N, L.B1, N);                                      // B1 = Ub^T B
       g.skip_dev = L.flags;               // skipped level: V = I, B1 is already Ua^T B
@@ -1146,7 +1136,7 @@ cudaError_t sym_eig(const double *G, int c, double *U, double *scratch, cudaStre
   int *state = L.flags + 8;
   cudaError_t e = cudaMemsetAsync(state, 0, kEigSteps * sizeof(int), st);
   if (e != cudaSuccess) return e;
-  e = eigvecs(G, c, L.U0, L.U1, 0.0, state, false, L, st);
+  e = eigvecs(G, c, L.U0, L.U1, 0.0, state, L, st);
   if (e != cudaSuccess) return e;
   return copy_f64(L.U0, U, (long long)c * c, st);
 }
