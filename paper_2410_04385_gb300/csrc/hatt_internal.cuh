@@ -143,6 +143,9 @@ bool gemm_split_applicable(const Gemm &g);
 size_t gemm_split_scratch_doubles(const Gemm &g);
 cudaError_t gemm_split(const Gemm &g, double *scratch, cudaStream_t st);
 cudaError_t split_error_word(int *value, bool clear);
+// FP64 products too small to fill the device (k_gemm_small.cu); no scratch.
+bool gemm_small_applicable(const Gemm &g);
+cudaError_t gemm_small(const Gemm &g, cudaStream_t st);
 // Error word set by a device wait that ran out (the kernel wrote NaN to its
 // outputs, freed its tensor memory and returned): read (synchronizing the
 // device) and clear it.

@@ -402,6 +402,7 @@ size_t gemm_scratch_doubles(const Gemm &g) {
   if (g.M <= 0 || g.N <= 0 || g.K <= 0) return 0;
   if (gemm_tc_supported(g)) return gemm_tc_scratch_doubles(g);
   if (gemm_split_applicable(g)) return gemm_split_scratch_doubles(g);
+  if (gemm_small_applicable(g)) return 0;
   const Launch L = plan(g);
   return L.ksplit > 1 ? (size_t)L.ksplit * g.batch * (size_t)g.M * g.N : 0;
 }
@@ -420,6 +421,12 @@ cudaError_t gemm_f64(const Gemm &g, double *scratch, cudaStream_t st) {
   if (gemm_split_applicable(g)) {                 // exact digits on the BF16 tensor cores
     const int slot = timer_begin(st);
     const cudaError_t e = gemm_split(g, scratch, st);
+    timer_end(slot, st, 2.0 * g.M * g.N * (double)g.K * g.batch, g.role);
+    return e;
+  }
+  if (gemm_small_applicable(g)) {
+    const int slot = timer_begin(st);
+    const cudaError_t e = gemm_small(g, st);
     timer_end(slot, st, 2.0 * g.M * g.N * (double)g.K * g.batch, g.role);
     return e;
   }
