@@ -242,6 +242,13 @@ constexpr int kMaxDevices = 64;
 cudaError_t refine_cluster_available(bool *ok);
 cudaError_t refine_cluster(const double *G, int c, double *U, double floor_norm, const int *skip,
                            cudaStream_t st);
+// The same with one block per column over the whole GPU, where
+// refine_columns_available says so: Ub (c x c) and xch (6 c doubles) scratch, bar
+// two zero words.
+cudaError_t refine_columns_available(int c, bool *ok);
+cudaError_t refine_columns(const double *G, int c, double *U, double *Ub, double *xch, double floor_norm,
+                           const int *skip, int *bar, cudaStream_t st);
+cudaError_t refine_health_word(int *value, bool clear);
 // Eigenvectors (columns of U, c x c row-major) of the symmetric c x c matrix G.
 size_t sym_eig_scratch_doubles(int c);
 cudaError_t sym_eig(const double *G, int c, double *U, double *scratch, cudaStream_t st);

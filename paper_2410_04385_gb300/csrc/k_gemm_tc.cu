@@ -276,12 +276,13 @@ TcLaunch tc_plan(const Gemm &g) {
 }  // namespace
 
 cudaError_t read_device_error(int *value) {
-  int split = 0, qr = 0, misc = 0;
+  int split = 0, qr = 0, misc = 0, refine = 0;
   cudaError_t e = cudaMemcpyFromSymbol(value, g_device_error, sizeof(int));
   if (e == cudaSuccess) e = split_error_word(&split, false);
   if (e == cudaSuccess) e = qr_health_word(&qr, false);
   if (e == cudaSuccess) e = misc_health_word(&misc, false);
-  if (e == cudaSuccess) *value = (*value != 0 || split != 0 ? kHealthTimeout : 0) | qr | misc;
+  if (e == cudaSuccess) e = refine_health_word(&refine, false);
+  if (e == cudaSuccess) *value = (*value != 0 || split != 0 ? kHealthTimeout : 0) | qr | misc | refine;
   return e;
 }
 
@@ -292,6 +293,7 @@ cudaError_t clear_device_error() {
   if (e == cudaSuccess) e = split_error_word(&split, true);
   if (e == cudaSuccess) e = qr_health_word(&split, true);
   if (e == cudaSuccess) e = misc_health_word(&split, true);
+  if (e == cudaSuccess) e = refine_health_word(&split, true);
   return e;
 }
 

@@ -733,7 +733,7 @@ level_prep_kernel(const double *G1, int c, int cap, const double *delta2, int le
     }
     if (!skip) scale[0] = s;
   }
-  if (tid < kEigSteps) eig_state[tid] = skip;
+  if (tid < kEigSteps + 2) eig_state[tid] = tid < kEigSteps ? skip : 0;
   const double inv_s = skip ? 0.0 : 1.0 / s;
   for (int e = tid; e < c * c; e += kThreads) {
     const int i = e / c, j = e % c;
@@ -988,7 +988,8 @@ size_t trunc_scratch_doubles(int la, int n, int lb, int lm, int nm) {
 // start, kRefineSteps Ogita-Aishima steps and kOrthSteps Newton-Schulz steps
 // in FP64, ping-ponging between Ua and Ub; the result lands in Ua.
 // state[j] != 0 turns step j into no-ops (state[0] also the FP32 start): the
-// caller clears state[0..kEigSteps) or sets it to skip everything, and a step
+// caller clears state[0..kEigSteps + 2) (the last two are a grid barrier's words)
+// or sets the first kEigSteps to skip everything, and a step
 // whose correction is below kConverged sets the flags of all later steps.
 static cudaError_t eigvecs(const double *A, int c, double *Ua, double *Ub, double floor_norm,
                            int *state, const Layout &L, cudaStream_t st) {
@@ -1001,6 +1002,8 @@ static cudaError_t eigvecs(const double *A, int c, double *Ua, double *Ub, doubl
   HATT_TRY(cudaGetLastError());
   if (c <= kEigFusedMax) {          // all refinement steps in one cluster launch
     bool ok = false;
+    HATT_TRY(refine_columns_available(c, &ok));
+    if (ok) return refine_columns(A, c, Ua, Ub, L.E, floor_norm, state, state + kEigSteps, st);
     HATT_TRY(refine_cluster_available(&ok));
     if (ok) return refine_cluster(A, c, Ua, floor_norm, state, st);
   }
@@ -1046,7 +1049,7 @@ cudaError_t trunc_step(double *Xk, int la, int n, int lb, double *Xkm1, int lm, 
 #define HATT_TRY(x) do { e = (x); if (e != cudaSuccess) return e; } while (0)
   int *state1 = L.flags + 8, *state2 = L.flags + 16;
   HATT_TRY(gemm_f64(g_gram(Xk, la, N, L.G), L.gs, st));
-  HATT_TRY(cudaMemsetAsync(state1, 0, kEigSteps * sizeof(int), st));
+  HATT_TRY(cudaMemsetAsync(state1, 0, (kEigSteps + 2) * sizeof(int), st));
   HATT_TRY(eigvecs(L.G, la, L.U0, L.U1, 0.0, state1, L, st));
   double *U = L.U0;
   HATT_TRY(gemm_f64(g_tn(U, Xk, la, N, N, L.B1, N), L.gs, st));
@@ -1134,7 +1137,7 @@ cudaError_t sym_eig(const double *G, int c, double *U, double *scratch, cudaStre
   if (c < 1 || c > kMaxSmall) return cudaErrorInvalidValue;
   Layout L = carve(scratch, c, 1, 1);
   int *state = L.flags + 8;
-  cudaError_t e = cudaMemsetAsync(state, 0, kEigSteps * sizeof(int), st);
+  cudaError_t e = cudaMemsetAsync(state, 0, (kEigSteps + 2) * sizeof(int), st);
   if (e != cudaSuccess) return e;
   e = eigvecs(G, c, L.U0, L.U1, 0.0, state, L, st);
   if (e != cudaSuccess) return e;
