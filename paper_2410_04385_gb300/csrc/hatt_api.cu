@@ -1237,6 +1237,7 @@ struct tt_batch_plan {
   int count = 0;
   std::vector<EnginePair> pairs;
   size_t ws_bytes = 0;
+  size_t ctl_off = 0;                // control words in the workspace
   size_t tables_off = 0;             // stage and task tables in the workspace
   int max_c = 1;
   std::vector<hatt::EngineStage> stages;
@@ -2012,25 +2013,36 @@ int tt_batched_plan_create(int32_t count, const tt_t *Y, const tt_t *Z, const tt
       load[l] += cost[j].flops;
     }
   }
+  // an engine pair has a region of its own (all run at the same time), the pairs
+  // of a stream share one (they run one after the other)
+  std::vector<size_t> lane_bytes(std::max(P->lanes, 1), 0);
   for (int j = 0; j < count; ++j) {
     EnginePair &ep = P->pairs[j];
-    ep.ws_off = off;
+    flag_ints += 4LL * ep.a.d;
     if (ep.lane >= 0) {
       ep.ws_bytes = (measure([&](Ws &ws) { return carve_hatt(ws, ep.a); },
                              [&](Runner &run, const HattBufs &b) { run_hatt(run, ep.a, b); }) + 255) &
                     ~(size_t)255;
-    } else {
-      ep.ws_bytes = eng_pair_bytes(ep.a);
-      for (int k = 0; k <= ep.a.d; ++k) P->max_c = std::max<int>(P->max_c, (int)ep.a.ell[k]);
+      lane_bytes[ep.lane] = std::max(lane_bytes[ep.lane], ep.ws_bytes);
+      continue;
     }
+    ep.ws_off = off;
+    ep.ws_bytes = eng_pair_bytes(ep.a);
     off += ep.ws_bytes;
-    flag_ints += 4LL * ep.a.d;
+    for (int k = 0; k <= ep.a.d; ++k) P->max_c = std::max<int>(P->max_c, (int)ep.a.ell[k]);
   }
+  std::vector<size_t> lane_off(lane_bytes.size());
+  for (size_t l = 0; l < lane_bytes.size(); ++l) {
+    lane_off[l] = off;
+    off += lane_bytes[l];
+  }
+  for (EnginePair &ep : P->pairs)
+    if (ep.lane >= 0) ep.ws_off = lane_off[ep.lane];
   // control words: head, status, per-pair completion counters, QR flags, then
   // the per-CTA profile words (all cleared every run)
   P->flags_bytes = ((2 + (size_t)count + (size_t)flag_ints) * sizeof(int) + 255) & ~(size_t)255;
   P->flags_bytes += (size_t)hatt::kMaxProfBlocks * hatt::kProfWords * sizeof(long long);
-  const size_t ctl_off = off;
+  const size_t ctl_off = P->ctl_off = off;
   off += P->flags_bytes;
   // count stages and the largest task count over the tile candidates with a
   // stand-in base address (pointers are formed, never dereferenced)
@@ -2076,7 +2088,7 @@ int tt_batched_plan_bind(tt_batch_plan *P, void *workspace, size_t workspace_byt
   if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) return from_cuda(cudaGetLastError());
   if (cs != cudaStreamCaptureStatusNone) return TT_ERR_ARG;        // synchronizes: not capturable
   char *ws = (char *)workspace;
-  const size_t ctl_off = P->pairs.back().ws_off + P->pairs.back().ws_bytes;
+  const size_t ctl_off = P->ctl_off;
   int *ctl = reinterpret_cast<int *>(ws + ctl_off);
   P->ws = ws;
   P->head = ctl;
