@@ -37,7 +37,8 @@ SKETCH_SEED = 9
 L2_FLUSH_BYTES = 256 << 20          # > 129 MB L2
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12   # SMs x FP64 FMA lanes/SM x 2 x max clock
 FP64_PEAK_NOTE = ("derived: 152 SMs x 2 FP64 FMA lanes/SM/clk x 2 flop x 2070 MHz = 1.259 TFLOP/s; "
-                  "a DFMA throughput loop measured 1.196 TFLOP/s on this GB300 pool")
+                  "a DFMA throughput loop measured 1.196 TFLOP/s; most of these products run on the "
+                  "tensor cores from exact 8-bit digits, so a fraction may exceed 1")
 
 
 GEMM_TIMING_STEPS = 3
@@ -637,8 +638,7 @@ def main():
     Zg = [torch.from_numpy(c).to(dev) for c in Z]
     h = binding.HadamardRecompressor(Yg, Zg, seed=SKETCH_SEED, **opts)
 
-    # a first call (the library times its GEMM tilings for shapes it has not
-    # run yet), then the launches and wall time of one eager call, then the
+    # a first call, then the launches and wall time of one eager call, then the
     # same sequence captured in a graph
     h.run()
     torch.cuda.synchronize()
@@ -758,7 +758,7 @@ def main():
         "e2e": {"value": world * 1000.0 / e2e_ms, "unit": UNIT, "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": d2h},
         "roofline": {"bound": "alu",
-                     "kernel": "gemm_f64_kernel, launches computing the HaTT contractions (HPCRL S1-S3, "
+                     "kernel": "FP64 products (digits on tcgen05, small, DFMA tiles), launches computing the HaTT contractions (HPCRL S1-S3, "
                                "C_k W, Q^T C_k, the two core-update stages)",
                      "achieved": meth_tflops, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                      "frac": meth_tflops / FP64_PEAK_TFLOPS, "traffic": traffic,
@@ -772,7 +772,7 @@ def main():
                      "timing": "CUDA events around every launch on its own stream (library kernel "
                                "timer), eager steps queued behind a GPU sleep",
                      "peak_source": FP64_PEAK_NOTE},
-        "gemm_aux": {"kernel": "gemm_f64_kernel, all other launches (truncation Gram matrices and "
+        "gemm_aux": {"kernel": "FP64 products, all other launches (truncation Gram matrices and "
                                "projections; the Cholesky QR computes its Gram matrix in its own "
                                "kernel)",
                      "launches_per_step": len(a_idx) / GEMM_TIMING_STEPS,
