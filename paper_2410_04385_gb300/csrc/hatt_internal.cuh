@@ -234,20 +234,14 @@ cudaError_t trunc_step(double *Xk, int la, int n, int lb, double *Xkm1, int lm, 
 // the calling thread while it issues its lanes.
 void set_host_sync(bool allowed);
 // FP64 refinement of a start U (c x c, in place) of the eigenvectors of the
-// symmetric c x c matrix G in one launch on a thread-block cluster
-// (k_refine.cu), for c <= kEigFusedMax; *skip != 0 leaves U untouched.
-// refine_cluster_available says whether the device can place the cluster.
+// symmetric c x c matrix G in one launch (k_refine.cu), for c <= kEigFusedMax:
+// Ub (c x c) and xch (6 c doubles) scratch, bar two zero words; *skip != 0 leaves U
+// untouched. refine_available says whether the device can place the cluster form.
 constexpr int kEigFusedMax = 96;
 constexpr int kMaxDevices = 64;
-cudaError_t refine_cluster_available(bool *ok);
-cudaError_t refine_cluster(const double *G, int c, double *U, double floor_norm, const int *skip,
-                           cudaStream_t st);
-// The same with one block per column over the whole GPU, where
-// refine_columns_available says so: Ub (c x c) and xch (6 c doubles) scratch, bar
-// two zero words.
-cudaError_t refine_columns_available(int c, bool *ok);
-cudaError_t refine_columns(const double *G, int c, double *U, double *Ub, double *xch, double floor_norm,
-                           const int *skip, int *bar, cudaStream_t st);
+cudaError_t refine_available(bool *ok);
+cudaError_t refine(const double *G, int c, double *U, double *Ub, double *xch, double floor_norm,
+                   const int *skip, int *bar, cudaStream_t st);
 cudaError_t refine_health_word(int *value, bool clear);
 // Eigenvectors (columns of U, c x c row-major) of the symmetric c x c matrix G.
 size_t sym_eig_scratch_doubles(int c);

@@ -910,6 +910,7 @@ __global__ void set_ranks_kernel(RankTable t, long long *ranks) {
 size_t eig_smem(int c) { return ((size_t)2 * c * (c + 1) + (size_t)c * c + 6 * (size_t)c) * sizeof(float); }
 
 struct Layout {
+  double *xch;                       // exchange words of the refinement
   double *G, *U0, *U1, *UtU, *T, *S, *E, *H, *V0, *V1, *B1, *e, *sigma, *K, *tmp, *gs, *scale;
   int *perm, *flags;
 };
@@ -936,12 +937,13 @@ Layout carve(double *base, int la, long long N, long long mrows) {
   L.perm = (int *)p; p += la;
   L.B1 = p; p += (size_t)la * N;
   L.tmp = p; p += (size_t)mrows * la;
+  L.xch = p; p += 6 * (size_t)la;
   L.gs = p;
   return L;
 }
 
 size_t carve_doubles(int la, long long N, long long mrows) {
-  return (size_t)11 * la * la + 13 + 3 * (size_t)la + (size_t)la * N + (size_t)mrows * la;
+  return (size_t)11 * la * la + 13 + 9 * (size_t)la + (size_t)la * N + (size_t)mrows * la;
 }
 
 Gemm g_gram(const double *B, int la, long long N, double *G) {
@@ -1000,12 +1002,10 @@ static cudaError_t eigvecs(const double *A, int c, double *Ua, double *Ub, doubl
   launch_k(eig_tridiag32_kernel, 1, kEigThreads, eig_smem(c), st, A, c, Ua, state);
   note_launch();
   HATT_TRY(cudaGetLastError());
-  if (c <= kEigFusedMax) {          // all refinement steps in one cluster launch
+  if (c <= kEigFusedMax) {          // all refinement steps in one launch
     bool ok = false;
-    HATT_TRY(refine_columns_available(c, &ok));
-    if (ok) return refine_columns(A, c, Ua, Ub, L.E, floor_norm, state, state + kEigSteps, st);
-    HATT_TRY(refine_cluster_available(&ok));
-    if (ok) return refine_cluster(A, c, Ua, floor_norm, state, st);
+    HATT_TRY(refine_available(&ok));
+    if (ok) return refine(A, c, Ua, Ub, L.xch, floor_norm, state, state + kEigSteps, st);
   }
   double *U = Ua, *Un = Ub;
   for (int it = 0; it < kEigSteps; ++it) {

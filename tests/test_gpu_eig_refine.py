@@ -34,7 +34,9 @@ def test_rank_cut_matches_the_oracle(c):
     Xo = ohatt.hadamard_recompress(Y, Z, **opts)
     lanes = binding.BatchRecompressor([(Yg, Zg, opts)], lanes=1)
     lanes.run()
-    for X in (binding.tt_hadamard_recompress(Yg, Zg, **opts), lanes.result(0)):
+    single = binding.tt_hadamard_recompress(Yg, Zg, **opts)
+    assert all(torch.equal(a, b) for a, b in zip(single, lanes.result(0)))   # both forms, bit for bit
+    for X in (single, lanes.result(0)):
         X = [x.cpu().numpy() for x in X]
         assert ott.ranks(X) == ott.ranks(Xo)
         assert ott.tt_diff_norm(X, Xo) <= 3e-10 * ott.tt_norm(Xo)
