@@ -211,7 +211,11 @@ int tt_round_plan(const tt_t *A, int64_t max_rank, double tol, int64_t *out_rank
  * of each vertical unfolding (left to right), then a right-to-left truncation
  * sweep with the same rule as tt_hadamard_recompress (max_rank cap, tol with
  * delta = tol * ||A|| / sqrt(d-1)). B is written like X above; all ranks of A
- * must be <= TT_MAX_SMALL_RANK. */
+ * must be <= TT_MAX_SMALL_RANK. The singular directions that B keeps have no sign of
+ * their own: it is the one the eigensolver arrives at, and where discarded energies
+ * lie below FP32 it follows the last bits of every sum before. Rounding therefore
+ * keeps one arithmetic (tt_gemm_autotune below); in tt_hadamard_recompress a
+ * direction's sign may change with the precision, the variant or the device. */
 int tt_round(const tt_t *A, int64_t max_rank, double tol, tt_t *B, void *workspace,
              size_t workspace_bytes, void *stream);
 
@@ -363,8 +367,18 @@ int tt_gemm(int32_t precision, int64_t M, int64_t N, int64_t K, int64_t batch, c
             const double *B, double *C, double alpha, void *workspace, size_t workspace_bytes,
             void *stream);
 
-/* Kept for its callers: FP64 products take their tilings from a cost model, and
- * nothing is timed. Returns TT_OK and changes nothing. */
+/* Product tuning of tt_round*, an implementation detail with no counterpart in the
+ * paper. Rounding keeps one arithmetic, so that its cores (and the signs of their
+ * singular directions) reproduce: DFMA products whose K split is part of it. The
+ * first time a product shape (sizes, operand layout) of at least 1e7 flops runs in
+ * a rounding on a stream that is not being captured, the library times its cost
+ * model's best tilings (~50 launches on the call's own operands and output) and
+ * keeps the fastest for every later launch of that shape in the process, including
+ * inside captured graphs. This synchronizes the caller's stream once per tuned shape
+ * and allocates nothing. A shape first met during a capture keeps the model's
+ * choice, and so do shapes beyond the first 256 tuned. tt_gemm_autotune(0) turns the
+ * timing off for shapes not yet run, 1 turns it on (the default). All other calls
+ * take their tilings from the model. Returns TT_OK; the setting is process-wide. */
 int tt_gemm_autotune(int32_t enable);
 
 /* Kernel timer, a diagnostic with no counterpart in the paper: between

@@ -226,7 +226,7 @@ def device_error() -> int:
 
 
 def gemm_autotune(enable: bool) -> None:
-    """Kept for its callers (tt_gemm_autotune): nothing is timed, nothing changes."""
+    """First-use timing of rounding's product tilings (tt_gemm_autotune); on by default."""
     _check("tt_gemm_autotune", load().tt_gemm_autotune(1 if enable else 0))
 
 

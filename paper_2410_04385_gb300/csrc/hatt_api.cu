@@ -889,6 +889,12 @@ struct SplitScope {
   ~SplitScope() { hatt::set_split_products(true); }
 };
 
+// One call with the arithmetic it has always had (set_kept_arithmetic).
+struct KeptScope {
+  KeptScope() { hatt::set_kept_arithmetic(true); }
+  ~KeptScope() { hatt::set_kept_arithmetic(false); }
+};
+
 // While a batch issues its lanes: the truncation sweep does not synchronize,
 // kernels are launched without programmatic serialization, and health bits go
 // to `status` (nullptr: the device error word).
@@ -1659,6 +1665,7 @@ int tt_round_ex_plan(const tt_t *A, int64_t max_rank, double tol, int32_t fixed_
   for (int k = 0; k <= a.d; ++k) out_rank_bound[k] = a.outb[k];
   a.A = nullptr;
   a.Bout = nullptr;
+  KeptScope kept;
   *workspace_bytes = measure([&](Ws &ws) { return carve_round(ws, a); },
                              [&](Runner &run, const RoundBufs &u) { run_round(run, a, u); });
   return TT_OK;
@@ -1692,6 +1699,7 @@ int tt_round_ex(const tt_t *A, int64_t max_rank, double tol, int32_t fixed_ranks
   a.Bout = B->cores;
   cudaStream_t strm = (cudaStream_t)stream;
   RoundBufs keep;
+  KeptScope kept;
   st = execute(workspace, workspace_bytes, strm,
                [&](Ws &ws) {
                  RoundBufs u = carve_round(ws, a);
@@ -1911,7 +1919,7 @@ int tt_gemm(int32_t precision, int64_t M, int64_t N, int64_t K, int64_t batch, c
 }
 
 int tt_gemm_autotune(int32_t enable) {
-  (void)enable;   // plans come from the cost model alone; the entry point stays for its callers
+  hatt::set_gemm_autotune(enable != 0);
   return TT_OK;
 }
 

@@ -135,7 +135,7 @@ size_t gemm_scratch_doubles(const Gemm &g);
 bool gemm_tc_supported(const Gemm &g);
 size_t gemm_tc_scratch_doubles(const Gemm &g);
 cudaError_t gemm_tc(const Gemm &g, double *scratch, int *counters, cudaStream_t st);
-// FP64 products on the BF16 tensor cores from exact digits of both operands
+// FP64 products on the FP16 tensor cores from exact digits of both operands
 // (k_gemm_split.cu); gemm_f64 dispatches to them by size.
 // set_split_products(false) keeps the calling thread on the DFMA kernels.
 void set_split_products(bool on);
@@ -146,6 +146,18 @@ cudaError_t split_error_word(int *value, bool clear);
 // FP64 products too small to fill the device (k_gemm_small.cu); no scratch.
 bool gemm_small_applicable(const Gemm &g);
 cudaError_t gemm_small(const Gemm &g, cudaStream_t st);
+// Calls that keep their arithmetic (TT rounding): the calling thread's products run
+// on the DFMA tiles in the K split that timing finds on a shape's first use, its QRs
+// in the one-column form and its eigenvector refinement in one chain per sum. The
+// FP32 start of an eigenbasis takes a direction's sign from the last bits of
+// everything before it once the spectrum falls below FP32 (a sum of tensors swept
+// from the right: 1e-11 of the largest energy at the second bond). With other sums
+// the rounded tensor is the same, but pairs of its cores come with some directions
+// negated (4 of 24 inputs of order 8, n = 64, rank 96 -> 24).
+void set_kept_arithmetic(bool on);
+bool kept_arithmetic();
+// First-use timing of those products' plans (on by default; see k_gemm.cu).
+void set_gemm_autotune(bool on);
 // Error word set by a device wait that ran out (the kernel wrote NaN to its
 // outputs, freed its tensor memory and returned): read (synchronizing the
 // device) and clear it.

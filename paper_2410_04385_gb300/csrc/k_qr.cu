@@ -746,6 +746,392 @@ qr_fused_kernel(double *S, int m, int c, long long ldS, double *G, double *Ut, d
   }
 }
 
+// ------------------------------------------------- the one-column form ---
+// The QR of calls that keep their arithmetic (set_kept_arithmetic): the grid form
+// with a factorization in every pass, one column per step, a warp per row in the
+// apply and a warp per entry in the sum of the shares. Its Q differs from the
+// other forms' in the last bits only, and costs more (600 x 30 56 us against 48,
+// 1600 x 50 97 and 78, 5760 x 90 314 and 265).
+
+// 1/x for x in [1e-30, 1e30] (a pivot pre-scaled by an even power of two):
+// an FP32 reciprocal seed (rcp.approx, relative error below 2^-22), then two
+// Newton-Raphson steps r <- r + r (1 - x r) in FP64, each two fused
+// multiply-adds (the error squares per step: 2^-22 -> 2^-44 -> FP64
+// rounding). Two dependent FP64 instructions fewer than rsqrt_scaled, and its
+// result is the multiplier 1/R_jj^2 the trailing update uses directly.
+__device__ __forceinline__ double rcp_scaled(double x) {
+  float f;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"((float)x));
+  double r = (double)f;
+  double e = fma(-x, r, 1.0);
+  r = fma(r, e, r);
+  e = fma(-x, r, 1.0);
+  return fma(r, e, r);
+}
+
+// Warp reduction of the three convergence statistics; lane 0 holds the
+// result. dev and dmax are maxima of non-negative doubles, taken on their bit
+// patterns (integer order equals numeric order there), which keeps them off
+// the FP64 unit.
+__device__ __forceinline__ void warp_stats(long long &dev, long long &dmax, double &tr) {
+  for (int o = 16; o > 0; o >>= 1) {
+    dev = max(dev, __shfl_xor_sync(0xffffffffu, dev, o));
+    dmax = max(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
+    tr += __shfl_xor_sync(0xffffffffu, tr, o);
+  }
+}
+
+// Pivot step of column j (thread 0 only): R_jj = sqrt(pivot), stored as
+// rinv2_j = 1/pivot, the multiplier of the trailing update, and the pivot
+// itself; 1/R_jj is formed at publication, for all j at once and off the
+// column chain. An exactly zero column of S (zero Gram diagonal) gets R_jj = 1,
+// which leaves Q_j = 0 and couples nothing; sending it to the shifted attempt
+// instead would make every pass shifted and leave ||Q^T Q - I|| at the shift
+// (~1e-11) on an otherwise benign S. A pivot not safely positive fails the
+// unshifted attempt; in the shifted attempt it sets the breakdown bit and is
+// clamped so that nothing divides by zero.
+// G is factorized scaled by sc = 2^-2k, which puts the largest Gram diagonal
+// near 1 (exact: a power of two), so every pivot above the failure floor is a
+// normal FP32 number and the chain carries no scaling; floor_piv and clamp
+// (the value a failed pivot takes) are scaled alike.
+__device__ __forceinline__ void chol_pivot(double *G, int ld, int j, const unsigned char *zero_col,
+                                           double floor_piv, double clamp, int attempt,
+                                           double *rinv2, double *pivots, unsigned char *fail,
+                                           int *health) {
+  if (zero_col[j]) {
+    rinv2[j] = 1.0;
+    pivots[j] = 1.0;
+    return;
+  }
+  double piv = G[j * ld + j];
+  if (!(piv > floor_piv)) {
+    if (attempt == 0) fail[j] = 1;
+    else atomicOr(health_word(health), kHealthBreakdown);
+    piv = clamp;
+  }
+  pivots[j] = piv;
+  rinv2[j] = (piv >= 1e-30 && piv <= 1e30) ? rcp_scaled(piv) : 1.0 / piv;
+}
+
+// Right-looking factorization with a one-column look-ahead: during the
+// trailing update for column j, warp 0 first updates row j + 1 and thread 0
+// takes the pivot of column j + 1 (the only serial step of the next column)
+// while the other warps update the rest, so each column costs one barrier and
+// the pivot's dependent FP64 chain overlaps the bulk of the update. Rows of R
+// are not scaled in place: the update subtracts (G_ji y_j^2) G_jl, and the
+// publication scales row j by y_j^2. G is read through L2 (__ldcg): in the
+// fused form other blocks of the same launch wrote it.
+__device__ __forceinline__ void chol_columns(const double *Gg, double *Ut_g, double *y_g, int c,
+                                             int m, int *flags, double *sm, int *health) {
+  const int ld = c + 1;
+  double *G = sm;                                   // c x ld, upper triangle is updated
+  __shared__ double s_red[3][kCholThreads / 32];
+  __shared__ double s_diag_max, s_trace, s_dev, s_sc, s_unsc;
+  __shared__ double s_rinv2[kMaxSmall];             // 1 / (sc R_jj^2)
+  __shared__ double s_piv[kMaxSmall];               // sc R_jj^2 (the scaled pivot)
+  __shared__ unsigned char s_zero[kMaxSmall];       // column j of S is exactly zero
+  __shared__ unsigned char s_failc[kMaxSmall];      // unshifted pivot j not safely positive
+  const int tid = threadIdx.x;
+  const int warp = tid >> 5, lane = tid & 31;
+  const int tx = tid % 16, ty = tid / 16;           // 16 x 16 grid (kCholThreads = 256)
+
+  // -- convergence test: G = I to working accuracy, except columns that are
+  // exactly zero (a zero column stays zero through every pass). The test is
+  // absolute on purpose: S of any scale (HaTT sketches of long chains reach
+  // 1e-20 and below) is never mistaken for a converged basis.
+  long long dev = 0, dmax = 0;          // bit patterns of non-negative doubles
+  double tr = 0.0;
+  int bad = 0;
+  const int n = c * c;
+  // entry e = i c + j of thread tid: (i, j) advanced by (di, dj) per step of
+  // kCholThreads entries, with a carry, instead of a division per entry
+  const int di = kCholThreads / c, dj = kCholThreads - (kCholThreads / c) * c;
+  int ii = tid / c, jj = tid - (tid / c) * c;
+  for (int e0 = tid; e0 < n; e0 += 4 * kCholThreads) {
+    double v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {         // four loads in flight per thread
+      const int e = e0 + q * kCholThreads;
+      v[q] = e < n ? __ldcg(Gg + e) : 0.0;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int e = e0 + q * kCholThreads;
+      if (e >= n) break;
+      const int i = ii, j = jj;
+      ii += di;
+      jj += dj;
+      if (jj >= c) {
+        jj -= c;
+        ++ii;
+      }
+      const long long bits = __double_as_longlong(fabs(v[q]));
+      bad |= bits >= 0x7ff0000000000000LL;                   // Inf or NaN
+      G[i * ld + j] = v[q];
+      if (i == j) {
+        s_zero[i] = (v[q] == 0.0);
+        dmax = max(dmax, bits);
+        tr += v[q];
+        if (v[q] != 0.0) dev = max(dev, __double_as_longlong(fabs(v[q] - 1.0)));
+      } else {
+        dev = max(dev, bits);
+      }
+    }
+  }
+  warp_stats(dev, dmax, tr);
+  if (lane == 0) {
+    s_red[0][warp] = __longlong_as_double(dev);
+    s_red[1][warp] = __longlong_as_double(dmax);
+    s_red[2][warp] = tr;
+  }
+  // a non-finite Gram matrix (a non-finite input core or intermediate): record
+  // it, leave S as it is and stop this QR (every later pass is a no-op)
+  if (__syncthreads_or(bad)) {
+    if (tid == 0) {
+      atomicOr(health_word(health), kHealthNonfinite);
+      flags[0] = 1;
+      flags[1] = 1;
+    }
+    return;
+  }
+  if (tid == 0) {
+    double d0 = 0.0, d1 = 0.0, d2 = 0.0;
+    for (int w = 0; w < kCholThreads / 32; ++w) {
+      d0 = fmax(d0, s_red[0][w]);
+      d1 = fmax(d1, s_red[1][w]);
+      d2 += s_red[2][w];
+    }
+    s_dev = d0;
+    s_diag_max = d1;
+    s_trace = d2;
+    // pivot scaling 2^-2k with the largest diagonal in [0.5, 2) after scaling;
+    // the exponent is read off the bits (frexp / ldexp are long sequences on
+    // this chain), with frexp / ldexp kept for subnormal or extreme values
+    const long long bits = __double_as_longlong(d1);
+    const int be = (int)((bits >> 52) & 0x7ff);
+    int ex = 0;
+    if (be > 0) ex = be - 1022;                 // d1 = m 2^ex, m in [0.5, 1)
+    else if (d1 > 0.0) frexp(d1, &ex);
+    const int k = ex / 2;
+    s_sc = (-2 * k + 1023 >= 1 && -2 * k + 1023 <= 2046)
+               ? __longlong_as_double((long long)(-2 * k + 1023) << 52) : ldexp(1.0, -2 * k);
+    s_unsc = (-k + 1023 >= 1 && -k + 1023 <= 2046)
+                 ? __longlong_as_double((long long)(-k + 1023) << 52) : ldexp(1.0, -k);
+  }
+  __syncthreads();
+  const double u = 1.1102230246251565e-16;
+  const double sc = s_sc, unsc = s_unsc;
+  if (s_dev <= 8.0 * c * u) {              // already orthonormal: nothing to apply
+    if (tid == 0) { flags[0] = 1; flags[1] = 1; }
+    return;
+  }
+  for (int i = ty; i < c; i += 16)         // the factorization runs on sc G
+    for (int j = tx; j < c; j += 16) G[i * ld + j] *= sc;
+
+  // -- Cholesky: first unshifted, then shifted if a pivot is not safely positive.
+  // A failed pivot of column j is recorded in s_failc[j] while column j - 1
+  // is updated and read by every thread after that column's barrier, so all
+  // threads leave the column loop at the same j.
+  for (int attempt = 0; attempt < 2; ++attempt) {
+    double shift = 0.0;
+    if (attempt == 1) {
+      shift = 11.0 * ((double)m * c + (double)c * (c + 1)) * u * s_trace;
+      if (!(shift > 0.0)) shift = 1e-300;
+      for (int e = tid; e < c * c; e += kCholThreads) {
+        const int i = e / c, j = e % c;
+        G[i * ld + j] = (__ldcg(Gg + e) + (i == j ? shift : 0.0)) * sc;
+      }
+      if (tid == 0) flags[3] += 1;
+    }
+    for (int j = tid; j < c; j += kCholThreads) s_failc[j] = 0;
+    __syncthreads();
+    const double floor_piv = (attempt == 0) ? (double)c * u * s_diag_max * sc : 0.0;
+    const double clamp = fmax(shift, 1e-300) * sc;
+    if (tid == 0) chol_pivot(G, ld, 0, s_zero, floor_piv, clamp, attempt, s_rinv2, s_piv, s_failc, health);
+    __syncthreads();
+    bool failed = false;
+    for (int j = 0; j < c; ++j) {
+      if (s_failc[j]) {
+        failed = true;
+        break;
+      }
+      const double y2 = s_rinv2[j];
+      const double *rowj = G + j * ld;
+      if (warp == 0 && j + 1 < c) {       // look-ahead: row j + 1, then its pivot
+        const int i = j + 1;
+        const double rji = rowj[i] * y2;
+        for (int l = i + lane; l < c; l += 32) G[i * ld + l] = fma(-rji, rowj[l], G[i * ld + l]);
+        __syncwarp();
+        if (lane == 0) chol_pivot(G, ld, i, s_zero, floor_piv, clamp, attempt, s_rinv2, s_piv, s_failc, health);
+      }
+      // trailing update of the rows below by warps 1..7 on a 14 x 16 grid:
+      // warp 0 carries the pivot chain and takes no share of it
+      if (warp > 0) {
+        const int bt = tid - 32, bx = bt % 16, by = bt / 16;
+        for (int i = j + 2 + by; i < c; i += 14) {
+          const double rji = rowj[i] * y2;
+          for (int l = i + bx; l < c; l += 16) G[i * ld + l] = fma(-rji, rowj[l], G[i * ld + l]);
+        }
+      }
+      __syncthreads();
+    }
+    if (!failed) break;
+    __syncthreads();                      // all reads of G and s_failc done before the retry
+  }
+
+  // -- publish R = D U~ as the unit upper triangle U~ (U~_jl = R_jl / R_jj =
+  // G_jl / G_jj with G the updated, scaled Gram row: the scale cancels) and
+  // y_j = 1 / R_jj; the apply
+  // kernel solves with them, so no serial triangular inverse is formed in
+  // this single block
+  for (int i = ty; i < c; i += 16) {
+    const double yi2 = s_rinv2[i];
+    for (int l = tx; l < c; l += 16)
+      Ut_g[i * c + l] = (l > i) ? G[i * ld + l] * yi2 : (l == i ? 1.0 : 0.0);
+  }
+  for (int i = tid; i < c; i += kCholThreads) {
+    double yi = 1.0;                      // 1 / R_ii (1 for an exactly zero column)
+    if (!s_zero[i]) {                     // the pivot is sc R_ii^2, sc = unsc^2
+      const double ps = s_piv[i];
+      yi = ((ps >= 1e-30 && ps <= 1e30) ? rsqrt_scaled(ps) : rsqrt_newton(ps)) * unsc;
+    }
+    y_g[i] = yi;
+  }
+  // this pass applies; ||G - I||_max <= 0.1/c puts every eigenvalue of G in
+  // [0.9, 1.1] (Gerschgorin): one more Cholesky QR pass orthonormalizes to
+  // working accuracy, so this pass is the last one. Written last: the
+  // read-modify-write would otherwise sit on the first pivot's path.
+  if (tid == 0) {
+    flags[1] = 0;
+    flags[2] += 1;
+    if (s_dev <= 0.1 / c) flags[0] = 1;
+  }
+}
+
+// Two rows at once, their chains interleaved (the same operations on each
+// row as trsm_row, so a row's result does not depend on its partner).
+template <int NS>
+__device__ __forceinline__ void trsm_row2(double (&x)[4], double (&z)[4], const double *Us, int c,
+                                          int lane) {
+#pragma unroll
+  for (int s0 = 0; s0 < NS; ++s0) {
+    const int lend = min(c, 32 * (s0 + 1));
+    for (int l = 32 * s0; l < lend; ++l) {
+      const double xl = __shfl_sync(0xffffffffu, x[s0], l & 31);
+      const double zl = __shfl_sync(0xffffffffu, z[s0], l & 31);
+      const double *u = Us + l * c;
+#pragma unroll
+      for (int s = s0; s < NS; ++s) {
+        const int col = lane + 32 * s;
+        if (col > l && col < c) {
+          const double uv = u[col];
+          x[s] = fma(-xl, uv, x[s]);
+          z[s] = fma(-zl, uv, z[s]);
+        }
+      }
+    }
+  }
+}
+
+__device__ __forceinline__ void apply_warp_rows(double *S, long long ldS, int c, const double *Us,
+                                                const double *ys, int r_first, int r_end, int r_step) {
+  const int lane = threadIdx.x & 31;
+  const int ns = (c + 31) / 32;          // column slots in use (c <= 128)
+  for (int r = r_first; r < r_end; r += 2 * r_step) {
+    double *row = S + (long long)r * ldS;
+    double *row2 = S + (long long)(r + r_step) * ldS;
+    const bool two = r + r_step < r_end;   // the warp's next row: solved alongside
+    double x[4], z[4];
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      const bool in = s < ns && lane + 32 * s < c;
+      x[s] = in ? row[lane + 32 * s] : 0.0;
+      z[s] = (in && two) ? row2[lane + 32 * s] : 0.0;
+    }
+    if (two) {
+      switch (ns) {
+        case 1: trsm_row2<1>(x, z, Us, c, lane); break;
+        case 2: trsm_row2<2>(x, z, Us, c, lane); break;
+        case 3: trsm_row2<3>(x, z, Us, c, lane); break;
+        default: trsm_row2<4>(x, z, Us, c, lane); break;
+      }
+    } else {
+      switch (ns) {
+        case 1: trsm_row<1>(x, Us, c, lane); break;
+        case 2: trsm_row<2>(x, Us, c, lane); break;
+        case 3: trsm_row<3>(x, Us, c, lane); break;
+        default: trsm_row<4>(x, Us, c, lane); break;
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      const int col = lane + 32 * s;
+      if (s < ns && col < c) {
+        row[col] = x[s] * ys[col];
+        if (two) row2[col] = z[s] * ys[col];
+      }
+    }
+  }
+}
+
+// Entry t of G summed over the nb shares by one warp: lanes over shares in
+// order, then a fixed shuffle tree; lane 0 writes G(i, j) and G(j, i).
+__device__ __forceinline__ void gram_entry(const double *part, int nb, int c, int t, double *G) {
+  const int lane = threadIdx.x & 31;
+  const int T = c * (c + 1) / 2;
+  constexpr int kPer = (kQrMaxBlocks + 31) / 32;
+  double sh[kPer];                        // all loads in flight, then summed in share order
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const int p = lane + 32 * k;
+    sh[k] = p < nb ? __ldcg(part + (long long)p * T + t) : 0.0;
+  }
+  double v = 0.0;
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) v += sh[k];
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lane == 0) {
+    int i, j;
+    upper_index(t, c, i, j);
+    G[i * c + j] = v;
+    G[j * c + i] = v;
+  }
+}
+
+template <int MAXQ>
+__global__ void __launch_bounds__(kCholThreads, 1)
+qr_columns_kernel(double *S, int m, int c, long long ldS, double *G, double *Ut, double *y,
+                  double *part, int *flags, int *health, long long spin_cap) {
+  pdl_enter();
+  extern __shared__ double sm[];
+  const int tid = threadIdx.x, warp = tid >> 5;
+  constexpr int kWarps = kCholThreads / 32;
+  const int nb = gridDim.x, bid = blockIdx.x;
+  const int per = (m + nb - 1) / nb;
+  const int r0 = min(m, bid * per), r1 = min(m, r0 + per);
+  const int T = c * (c + 1) / 2;
+  GramSlots<MAXQ> g;
+  gram_slots(c, g);
+  int *bar = flags + 4;
+  int epoch = 0;
+  for (int pass = 0; pass < kPasses; ++pass) {
+    gram_share(S, ldS, c, r0, r1, g, part + (long long)bid * T, sm);
+    if (!grid_barrier(bar, epoch, spin_cap)) return;
+    for (int t = bid * kWarps + warp; t < T; t += nb * kWarps) gram_entry(part, nb, c, t, G);
+    if (!grid_barrier(bar, epoch, spin_cap)) return;
+    if (bid == 0) chol_columns(G, Ut, y, c, m, flags, sm, health);
+    if (!grid_barrier(bar, epoch, spin_cap)) return;
+    const int done = __ldcg(flags), skip = __ldcg(flags + 1);
+    if (skip) return;                      // orthonormal already (or a non-finite G)
+    for (int e = tid; e < c * c; e += kCholThreads) sm[e] = __ldcg(Ut + e);
+    for (int e = tid; e < c; e += kCholThreads) sm[c * c + e] = __ldcg(y + e);
+    __syncthreads();
+    apply_warp_rows(S, ldS, c, sm, sm + c * c, r0 + warp, r1, kWarps);
+    if (done) return;                      // this pass was the last one
+    if (!grid_barrier(bar, epoch, spin_cap)) return;
+  }
+}
+
 // SMs and cooperative-launch support of the current device, cached per
 // device (0 SMs: unknown device).
 void device_info(int &sms, bool &coop) {
@@ -779,14 +1165,16 @@ bool cluster_sized(int m, int c) { return (long long)m * (c * (c + 1) / 2) <= kC
 
 // Blocks (Gram shares) of a QR of m rows: at least kQrMinRows rows each, at
 // most one per SM (the grid form keeps every block resident).
-int qr_blocks(int m, int c, int sms) {
+int grid_blocks(int m, int sms) {
   const int want = (m + kQrMinRows - 1) / kQrMinRows;
-  if (cluster_sized(m, c)) {
-    int nb = kClusterBlocks;
-    while (nb / 2 >= want) nb /= 2;
-    return nb;
-  }
   return std::max(1, std::min({want, std::max(sms, 1), kQrMaxBlocks}));
+}
+int qr_blocks(int m, int c, int sms) {
+  if (!cluster_sized(m, c)) return grid_blocks(m, sms);
+  const int want = (m + kQrMinRows - 1) / kQrMinRows;
+  int nb = kClusterBlocks;
+  while (nb / 2 >= want) nb /= 2;
+  return nb;
 }
 
 // Test hooks, read once: HATT_QR_FORM=steps makes single calls use the
@@ -859,6 +1247,25 @@ cudaError_t qr_inplace(double *S, int m, int c, long long ldS, double *scratch, 
   const bool small = c <= 64;               // the kQrSlots64 instantiations
   const bool cluster = cluster_sized(m, c) && qr_spin_cap() == kQrSpinCap;
   cudaError_t e = cudaSuccess;
+  if (kept_arithmetic() && coop && programmatic_launch() && !force_qr_steps()) {
+    auto kernel = small ? qr_columns_kernel<kQrSlots64> : qr_columns_kernel<kQrMaxSlots>;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fused_smem(kMaxSmall));
+    if (e == cudaSuccess) e = cudaMemsetAsync(flags, 0, 6 * sizeof(int), st);
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.numAttrs = 1;
+    cfg.gridDim = dim3(grid_blocks(m, sms));
+    cfg.blockDim = dim3(kCholThreads);
+    cfg.dynamicSmemBytes = fused_smem(c);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    e = cudaLaunchKernelEx(&cfg, kernel, S, m, c, ldS, G, Ut, y, part, flags, health_target(), qr_spin_cap());
+    note_launch();
+    return e;
+  }
   if (!force_qr_steps() && (cluster || (coop && programmatic_launch()))) {
     auto kernel = cluster ? (small ? qr_fused_kernel<kQrSlots64, true> : qr_fused_kernel<kQrMaxSlots, true>)
                           : (small ? qr_fused_kernel<kQrSlots64, false> : qr_fused_kernel<kQrMaxSlots, false>);

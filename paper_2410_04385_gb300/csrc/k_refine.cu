@@ -22,9 +22,12 @@
 // the dependent FP64 chains, above the FP64 unit of c SMs (cluster: of 16).
 // Measured (us, grid and a cluster kernel): c = 10 27 and 34, 18 to 30 31 and 42,
 // 34 51 and 69, 50 41 and 59, 90 79 and 215, 96 80 and 237.
+#include <cooperative_groups.h>
 #include <algorithm>
 #include <mutex>
 #include "hatt_internal.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace hatt {
 namespace {
@@ -255,18 +258,197 @@ refine_columns_kernel(const double *G, int c, double *U, double *Ub, double *xch
   }
 }
 
+// The refinement of calls that keep their arithmetic (set_kept_arithmetic): CTA r
+// of a cluster owns a slice of the columns of R, S and the new U, every CTA holds G
+// and U whole in shared memory, and slices and per-CTA norms travel through
+// distributed shared memory, three cluster barriers per step. Sums run over k in
+// one chain, so the results differ from the kernel's above in the last bits.
+// Bound by the FP64 units of its 16 SMs (c = 90: 215 us, above 79).
+constexpr int kThreadsE = 512;
+
+// Block-wide sum / max of one double per thread. Only the warp shuffles run
+// in every thread; the final combination of the per-warp values runs in
+// thread 0 and is broadcast through shared memory: on GB300 every FP64
+// instruction that all 512 threads execute costs the SM ~256 clocks.
+__device__ __forceinline__ double blk_reduce(double v, double *red, bool is_max) {
+  for (int o = 16; o > 0; o >>= 1) {
+    const double x = __shfl_xor_sync(0xffffffffu, v, o);
+    v = is_max ? fmax(v, x) : v + x;
+  }
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  __syncthreads();
+  if (l == 0) red[w] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = red[0];
+    for (int i = 1; i < (int)(blockDim.x >> 5); ++i) t = is_max ? fmax(t, red[i]) : t + red[i];
+    red[32] = t;
+  }
+  __syncthreads();
+  return red[32];
+}
+
+// U (c x c, row-major, device) holds the start on entry and the refined
+// eigenvectors on return; *skip != 0 leaves it untouched.
+__global__ void __launch_bounds__(kThreadsE, 1)
+oa_cluster_kernel(const double *G, int c, double *Uout, double floor_norm, const int *skip) {
+  pdl_enter();
+  if (skip && *skip) return;           // every CTA reads the same word
+  cg::cluster_group cl = cg::this_cluster();
+  const int P = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const int w = (c + P - 1) / P;
+  const int j0 = min(c, rank * w), j1 = min(c, j0 + w), wl = j1 - j0;
+  extern __shared__ __align__(16) double sm[];
+  double *Gs = sm;                     // c x c
+  double *Us = Gs + c * c;             // c x c
+  double *lam = Us + c * c;            // c
+  double *part = lam + c;              // 3 x kMaxCluster
+  double *work = part + 3 * kMaxCluster;
+  double *Rs = work, *Ts = Rs + c * w, *Ss = Ts + c * w, *Ns = Ss + c * w;
+  __shared__ double red[33];
+  __shared__ double s_gn, s_delta, s_inv, s_stop;
+
+  double g2 = 0.0;
+  for (int e = tid; e < c * c; e += nt) {
+    const double v = G[e];
+    Gs[e] = v;
+    Us[e] = Uout[e];
+    g2 = fma(v, v, g2);
+  }
+  g2 = blk_reduce(g2, red, false);
+  if (tid == 0) s_gn = sqrt(g2);
+  cl.sync();                           // every CTA has started and loaded U
+  const double u = 1.1102230246251565e-16;
+  for (int it = 0; it < kRefine + kOrth; ++it) {
+    const bool orth = it >= kRefine;
+    // R = I - U^T U and T = G U on the own columns, then S = U^T T
+    for (int e = tid; e < c * wl; e += nt) {
+      const int i = e / wl, jj = e - i * wl, j = j0 + jj;
+      double r = 0.0, t = 0.0;
+      if (orth) {
+        for (int k = 0; k < c; ++k) r = fma(Us[k * c + i], Us[k * c + j], r);
+      } else {
+        for (int k = 0; k < c; ++k) {
+          const double ukj = Us[k * c + j];
+          r = fma(Us[k * c + i], ukj, r);
+          t = fma(Gs[i * c + k], ukj, t);
+        }
+      }
+      Rs[i * w + jj] = ((i == j) ? 1.0 : 0.0) - r;
+      Ts[i * w + jj] = t;
+    }
+    __syncthreads();
+    if (!orth) {
+      for (int e = tid; e < c * wl; e += nt) {
+        const int i = e / wl, jj = e - i * wl;
+        double s = 0.0;
+        for (int k = 0; k < c; ++k) s = fma(Us[k * c + i], Ts[k * w + jj], s);
+        Ss[i * w + jj] = s;
+      }
+      __syncthreads();
+      for (int jj = tid; jj < wl; jj += nt) {      // l_j to every CTA
+        const int j = j0 + jj;
+        const double l = Ss[j * w + jj] / (1.0 - Rs[j * w + jj]);
+        for (int q = 0; q < P; ++q) cl.map_shared_rank(lam, q)[j] = l;
+      }
+      double r2 = 0.0, s2 = 0.0;
+      for (int e = tid; e < c * wl; e += nt) {
+        const int i = e / wl, jj = e - i * wl, j = j0 + jj;
+        const double r = Rs[i * w + jj];
+        double sd = Ss[i * w + jj];
+        if (i == j) sd -= Ss[j * w + jj] / (1.0 - Rs[j * w + jj]);
+        r2 = fma(r, r, r2);
+        s2 = fma(sd, sd, s2);
+      }
+      r2 = blk_reduce(r2, red, false);
+      s2 = blk_reduce(s2, red, false);
+      if (tid == 0)
+        for (int q = 0; q < P; ++q) {
+          double *pr = cl.map_shared_rank(part, q);
+          pr[2 * rank] = r2;
+          pr[2 * rank + 1] = s2;
+        }
+      cl.sync();
+      if (tid == 0) {
+        double R2 = 0.0, S2 = 0.0;
+        for (int q = 0; q < P; ++q) {
+          R2 += part[2 * q];
+          S2 += part[2 * q + 1];
+        }
+        const double gn = s_gn;
+        s_delta = fmax(2.0 * (sqrt(S2) + gn * sqrt(R2)),
+                       64.0 * c * u * (floor_norm > 0.0 ? floor_norm : gn));
+        s_inv = gn > 0.0 ? 1.0 / gn : 1.0;
+      }
+      __syncthreads();
+    }
+    const double delta = s_delta, inv = s_inv;
+    // E (over R, in place), then the new columns U (I + E)
+    double emax = 0.0;
+    for (int e = tid; e < c * wl; e += nt) {
+      const int i = e / wl, jj = e - i * wl, j = j0 + jj;
+      const double r = Rs[i * w + jj];
+      double E = 0.5 * r;
+      if (!orth && i != j && fabs(lam[i] - lam[j]) > delta) {
+        const float num = (float)(fma(lam[j], r, Ss[i * w + jj]) * inv);
+        const float den = (float)((lam[j] - lam[i]) * inv);
+        const float qv = __fdividef(num, den);
+        if (fabsf(qv) <= 0.1f) E = (double)qv;
+      }
+      emax = fmax(emax, fabs(E));
+      Rs[i * w + jj] = E;
+    }
+    __syncthreads();
+    for (int e = tid; e < c * wl; e += nt) {
+      const int i = e / wl, jj = e - i * wl, j = j0 + jj;
+      double v = Us[i * c + j];
+      for (int k = 0; k < c; ++k) v = fma(Us[i * c + k], Rs[k * w + jj], v);
+      Ns[i * w + jj] = v;
+    }
+    emax = blk_reduce(emax, red, true);
+    if (tid == 0)
+      for (int q = 0; q < P; ++q) cl.map_shared_rank(part, q)[2 * kMaxCluster + rank] = emax;
+    cl.sync();                         // every CTA has finished reading U
+    for (int q = 0; q < P; ++q) {
+      double *dst = cl.map_shared_rank(Us, q);
+      for (int e = tid; e < c * wl; e += nt) {
+        const int i = e / wl, jj = e - i * wl;
+        dst[i * c + j0 + jj] = Ns[i * w + jj];
+      }
+    }
+    cl.sync();
+    if (tid == 0) {
+      double mx = 0.0;
+      for (int q = 0; q < P; ++q) mx = fmax(mx, part[2 * kMaxCluster + q]);
+      s_stop = (mx <= kStepConverged) ? 1.0 : 0.0;
+    }
+    __syncthreads();
+    if (s_stop != 0.0) break;          // the same decision in every CTA
+  }
+  for (int e = tid; e < c * wl; e += nt) {
+    const int i = e / wl, jj = e - i * wl;
+    Uout[i * c + j0 + jj] = Us[i * c + j0 + jj];
+  }
+}
+
 int cluster_size_for(int c) { return c >= 32 ? 16 : (c >= 8 ? 8 : 1); }
+
+size_t refine_smem(int c, int P) {
+  const int w = (c + P - 1) / P;
+  return ((size_t)2 * c * c + c + 3 * kMaxCluster + (size_t)4 * c * w) * sizeof(double);
+}
 
 size_t columns_smem(int c, int blocks) {
   const int w = (c + blocks - 1) / blocks;
   return ((size_t)2 * c * (c | 1) + (size_t)(2 * kMaxGroups + 2 + 3 * w) * c) * sizeof(double);
 }
 
-// Largest cluster (16, else 8) the device can place with the kernel's shared
+// Largest cluster (16, else 8) the device can place with the kernels' shared
 // memory, and its SMs if it launches cooperative grids, found once per device.
 struct Device {
   bool known = false;
-  int cluster = 0, coop_sms = 0;
+  int cluster = 0, kept_cluster = 0, coop_sms = 0;
 };
 Device g_device[kMaxDevices];
 std::mutex g_device_mu;
@@ -290,28 +472,34 @@ cudaError_t device_info(Device *out) {
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(refine_columns_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)columns_smem(kEigFusedMax, kEigFusedMax));
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(oa_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)refine_smem(kEigFusedMax, kMaxCluster));
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(oa_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     D.coop_sms = coop ? sms : 0;
-    for (int P : {kMaxCluster, 8}) {
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = P;
-      attr[0].val.clusterDim.y = 1;
-      attr[0].val.clusterDim.z = 1;
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(P);
-      cfg.blockDim = dim3(kTG);
-      cfg.dynamicSmemBytes = columns_smem(kEigFusedMax, P);
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      int clusters = 0;
-      if (cudaOccupancyMaxActiveClusters(&clusters, refine_columns_kernel<true>, &cfg) == cudaSuccess &&
-          clusters > 0) {
-        D.cluster = P;
-        break;
+    auto largest = [](auto kernel, int threads, size_t (*smem)(int, int)) {
+      for (int P : {kMaxCluster, 8}) {
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = P;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(P);
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = smem(kEigFusedMax, P);
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int clusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters > 0) return P;
+        cudaGetLastError();
       }
-      cudaGetLastError();
-    }
+      return 0;
+    };
+    D.cluster = largest(refine_columns_kernel<true>, kTG, columns_smem);
+    D.kept_cluster = largest(oa_cluster_kernel, kThreadsE, refine_smem);
     D.known = true;
   }
   *out = D;
@@ -323,7 +511,7 @@ cudaError_t device_info(Device *out) {
 cudaError_t refine_available(bool *ok) {
   Device D;
   const cudaError_t e = device_info(&D);
-  *ok = e == cudaSuccess && D.cluster > 0;
+  *ok = e == cudaSuccess && (kept_arithmetic() ? D.kept_cluster : D.cluster) > 0;
   return e;
 }
 
@@ -333,9 +521,10 @@ cudaError_t refine(const double *G, int c, double *U, double *Ub, double *xch, d
   Device D;
   cudaError_t e = device_info(&D);
   if (e != cudaSuccess) return e;
-  if (D.cluster == 0) return cudaErrorNotSupported;
-  const bool grid = programmatic_launch() && c >= kColumnsMin && D.coop_sms >= c;
-  const int blocks = grid ? c : std::min(cluster_size_for(c), D.cluster);
+  const bool kept = kept_arithmetic();
+  if ((kept ? D.kept_cluster : D.cluster) == 0) return cudaErrorNotSupported;
+  const bool grid = !kept && programmatic_launch() && c >= kColumnsMin && D.coop_sms >= c;
+  const int blocks = grid ? c : std::min(cluster_size_for(c), kept ? D.kept_cluster : D.cluster);
   cudaLaunchAttribute attr[2];
   cudaLaunchConfig_t cfg = {};
   if (grid) {
@@ -352,10 +541,15 @@ cudaError_t refine(const double *G, int c, double *U, double *Ub, double *xch, d
     cfg.numAttrs = programmatic_launch() ? 2 : 1;
   }
   cfg.gridDim = dim3(blocks);
-  cfg.blockDim = dim3(kTG);
-  cfg.dynamicSmemBytes = columns_smem(c, blocks);
+  cfg.blockDim = dim3(kept ? kThreadsE : kTG);
+  cfg.dynamicSmemBytes = kept ? refine_smem(c, blocks) : columns_smem(c, blocks);
   cfg.stream = st;
   cfg.attrs = attr;
+  if (kept) {
+    e = cudaLaunchKernelEx(&cfg, oa_cluster_kernel, G, c, U, floor_norm, skip);
+    note_launch();
+    return e;
+  }
   e = cudaLaunchKernelEx(&cfg, grid ? refine_columns_kernel<false> : refine_columns_kernel<true>, G, c, U, Ub,
                          xch, floor_norm, skip, bar);
   note_launch();
