@@ -72,12 +72,15 @@ typedef struct {
  * low-precision modes have no counterpart in it. */
 typedef enum {
   TT_FP64 = 0,           /* binary64 throughout. Products that are large enough run on the FP16
-                            tensor cores without loss: each operand entry is cut into eight
-                            8-bit digits of a 62-bit integer (its row or column scaled by a
-                            power of two), digit products are summed exactly in FP32 over
-                            at most 128 terms, and each such sum is rounded once to
-                            binary64; the error is below that of a chain of binary64
-                            fused multiply-adds, which smaller products use */
+                            tensor cores: each operand entry is cut into eight 8-bit digits
+                            of a 62-bit integer (its row or column scaled by a power of
+                            two), digit products are summed exactly in FP32 over at most
+                            128 terms, and each such sum is rounded once to binary64. A sum
+                            for which the digits may hold less than a chain of binary64
+                            fused multiply-adds would (terms far below the product of the
+                            row's and the column's largest entries) is formed by such
+                            a chain instead: the error of every element stays within a
+                            few K 2^-53 sum |a||b|. Smaller products are such chains */
   TT_MIXED_FP32 = 1,     /* HPCRL-1 products: FP32 operands, FP32 accumulation */
   TT_MIXED_TF32 = 2,     /* HPCRL-1 products: TF32 operands, FP32 accumulation */
   TT_MIXED_BF16 = 3,     /* HPCRL-1 products: BF16 operands, FP32 accumulation */

@@ -33,11 +33,21 @@
 //   6. the 8 level sums of an output are exact integers; they are combined in
 //      integer arithmetic to T = sum_l L_l 256^(7-l), rounded once to a double,
 //      scaled by 2^(e_i + f_j) and added to the output tile in shared memory.
-// The dropped digit products weigh 2^-62 (2^-60 if chunks follow) of
-// (row max)(column max) each, the digits' truncation as much: the error is
-// below that of the FP64 FMA chain it replaces (K roundings of 2^-53 of the
-// running sum). A row
-// or column with a non-finite entry gives NaN in all its outputs.
+// Dropped digit products and truncation leave at most 2^-58.8 of S = 2^(e_i + f_j)
+// per term (2^-62 rms). Against the rounding of an FP64 chain, 2^-53 sum |a||b|, that
+// is small unless the sum is far below S: where a row's large entries meet zeros or
+// small entries of the column (block-structured factors of a sum of tensors,
+// alternately graded rows). So
+//   7. an output keeps its digit sum only if sum |a||b| >= 2^-7.7 S is certain:
+//      because the sum itself is that large, or one term has both its entries at
+//      4.5 / 64 of their scales or more (one bit per entry, an AND of two 128-bit
+//      masks per output). Any other output's group is summed again from the
+//      operands in FP64 (fallback). Then a term's error is at most 3.5 2^-53 of
+//      sum |a||b|, 0.4 2^-53 rms, and terms' errors are independent: no element is
+//      worse than a chain's bound, whatever the operands' grading.
+//      Outputs summed twice: none of Gaussian factors, 0.1% where entries are
+//      products of two or three Gaussians.
+// A row or column with a non-finite entry gives NaN in all its outputs.
 //
 // Bound: issue slots of the conversion (about 40 instructions per operand
 // entry) and of the level combination (about 60 per output and group); FP64
@@ -73,6 +83,7 @@ constexpr int kLdRaw = kRows + 2;        // raw tiles are [k][row]; 4 k apart = 
 constexpr int kABytes = kDig * kRows * kKc * 2;
 constexpr int kNonfinite = 1 << 20;      // row / column exponent of a non-finite entry
 constexpr int kEmpty = -(1 << 20);       // exponent of an all-zero row / column
+constexpr int kSure = 5200;              // 2^20 2^-7.66: a sum this large is no cancelled one
 constexpr long long kSplitWaitLimit = 2000000;
 
 // Shared memory of the NT-column form: digits of both operands, raw tiles,
@@ -222,6 +233,50 @@ __device__ __forceinline__ unsigned long long digits(double x, int base) {
   return m + 0x8080808080808080ull;
 }
 
+// One bit per entry of u (four consecutive k, bits 0 to 3): its leading digit is
+// 5 or more, i.e. the entry is at least 4.5 / 64 of the row's scale. The biased
+// leading bytes are 128 to 192.
+__device__ __forceinline__ uint32_t large_bits(const unsigned long long (&u)[4]) {
+  const uint32_t a = __byte_perm((uint32_t)(u[0] >> 32), (uint32_t)(u[1] >> 32), 0x0073);
+  const uint32_t b = __byte_perm((uint32_t)(u[2] >> 32), (uint32_t)(u[3] >> 32), 0x0073);
+  const uint32_t w = __byte_perm(a, b, 0x5410) & 0x7F7F7F7Fu;
+  return ((((w + 0x7B7B7B7Bu) >> 7) & 0x01010101u) * 0x10204080u) >> 28;
+}
+
+// Adds a group's terms of the outputs marked in todo (bit t: column c4 + t % 4 +
+// t / 4 * 16 of this lane's row) to them in FP64: r the row's first term in the
+// group, cols + coff[column] the column's. Few outputs of a column: the lanes share
+// the terms of one after the other; many: each lane its own.
+constexpr int kLaneFallback = 8;
+__device__ __noinline__ void fallback(uint32_t todo, const double *r, long long sr, const double *cols,
+                                      const long long *coff, long long sc, int n, double *out, int c4) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t any = __reduce_or_sync(0xffffffffu, todo);
+#pragma unroll 1
+  for (uint32_t rest = any; rest != 0; rest &= rest - 1) {
+    const int t = __ffs(rest) - 1, col = c4 + t % 4 + t / 4 * (kThreadsS / 32);
+    const bool mine = todo >> t & 1u;
+    uint32_t lanes = __ballot_sync(0xffffffffu, mine);
+    const double *c = cols + coff[col];
+    if (__popc(lanes) >= kLaneFallback) {
+      double v = 0.0;
+#pragma unroll 8
+      for (int k = 0; k < n; ++k) v = fma(r[k * sr], c[k * sc], v);
+      if (mine) out[col] += v;
+      continue;
+    }
+    for (; lanes != 0; lanes &= lanes - 1) {
+      const int l = __ffs(lanes) - 1;
+      const double *rl = reinterpret_cast<const double *>(
+          __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(r), l));
+      double v = 0.0;
+      for (int k = lane; k < n; k += 32) v = fma(rl[k * sr], c[k * sc], v);
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane == l) out[col] += v;
+    }
+  }
+}
+
 // Digits of four consecutive k of one row as FP16 (exact integers): 8 bytes per
 // digit slice at dst + p * slice. The bytes of two k are interleaved; a byte
 // b = d + 128 under 0x64 is the FP16 number 1024 + b, and one packed
@@ -264,8 +319,8 @@ __device__ __noinline__ double scaled(long long q, int s) {
 // exact integers in FP32 (|L_l| <= l 2^21, |L_0| <= 2^19 over 128 terms), T is
 // formed and rounded (once) in integer arithmetic, mostly additions and shifts:
 // a 32 x 32 -> 64 multiply-add runs at 24 lanes per clock, an addition at 128.
-// ex = e_i + f_j of the row and column exponents.
-__device__ __forceinline__ double combine(const uint32_t (&L)[kDig], int ex) {
+// ex = e_i + f_j of the row and column exponents; t3: the sum in units of 2^-20 S.
+__device__ __forceinline__ double combine(const uint32_t (&L)[kDig], int ex, int32_t &t3) {
   // levels 0..2 stay within 2^22: 1.5 2^23 + L holds L in its low bits; the
   // others take a conversion (a pipe of its own)
   int32_t v[kDig];
@@ -279,7 +334,7 @@ __device__ __forceinline__ double combine(const uint32_t (&L)[kDig], int ex) {
   const int32_t x5 = v[5] + (x6 >> 8);
   const int32_t x4 = v[4] + (x5 >> 8);
   const int32_t t2 = v[2] * 256 + v[3] + (x4 >> 8);
-  const int32_t t3 = v[0] * 256 + v[1] + (t2 >> 16);
+  t3 = v[0] * 256 + v[1] + (t2 >> 16);
   const uint32_t s = (uint32_t)(t3 >> 31);           // sign: 0 or ~0
   // |T| = a 2^64 + b 2^32 + c
   uint32_t c = __byte_perm(__byte_perm((uint32_t)v[7], (uint32_t)x6, 0x0040),
@@ -318,6 +373,8 @@ gemm_split_kernel(const SplitArgs g) {
   __shared__ int s_mr[2][kRows], s_mc[2][NT];          // largest exponents of a chunk, by its parity
   __shared__ int s_er[kRows], s_ec[NT];                // scales of the group
   __shared__ __align__(16) int s_sh[kKc];              // exponent moved from rows to columns at each k
+  // large entries of the group, a bit per k (large_bits), a word per chunk
+  __shared__ __align__(16) uint32_t s_lr[kRows][kGroup], s_lc[NT][kGroup];
   __shared__ uint32_t s_taddr;
   __shared__ __align__(8) uint64_t s_bar;
   __shared__ int s_odd, s_go;                  // s_go: 0 / 1 first / later chunk of a group, 2 stop
@@ -429,7 +486,7 @@ gemm_split_kernel(const SplitArgs g) {
   // room above the first chunk's largest entries for those of the group's
   // other chunks; none where there are no others
   const int margin = kend - kbeg > kKc ? 1 : 0;
-  int par = 0, grp = 0;
+  int par = 0, grp = 0, kgrp = kbeg;     // kgrp: the group's first term
 #pragma unroll 1
   for (int k0 = kbeg;; k0 += kKc, par ^= 1) {
     const bool live = k0 < kend;         // false once: only the last group's sums are left
@@ -513,6 +570,11 @@ gemm_split_kernel(const SplitArgs g) {
         // add the level sums to the output tile
         const int orow = 32 * (warp & 3) + lane;
         const int eri = s_er[orow];
+        uint4 lrow = *reinterpret_cast<const uint4 *>(s_lr[orow]);
+        if (grp < 4) lrow.w = 0;         // chunks the group does not have
+        if (grp < 3) lrow.z = 0;
+        if (grp < 2) lrow.y = 0;
+        uint32_t todo = 0;               // this thread's outputs that need the FP64 sum
         const uint32_t td = s_taddr + ((uint32_t)(32 * (warp & 3)) << 16);
 #pragma unroll 1
         for (int c4 = 4 * (warp >> 2); c4 < nc; c4 += kThreadsS / 32) {
@@ -528,9 +590,17 @@ gemm_split_kernel(const SplitArgs g) {
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             const int ecj = s_ec[c4 + j];
-            v[j] = combine(L[j], eri + ecj);
-            if (min(eri, ecj) < kEmpty / 2) v[j] = 0.0;
-            if (max(eri, ecj) > kNonfinite / 2) v[j] = __longlong_as_double(0x7FF8000000000000LL);
+            int32_t t3;
+            v[j] = combine(L[j], eri + ecj, t3);
+            const bool empty = min(eri, ecj) < kEmpty / 2, inf = max(eri, ecj) > kNonfinite / 2;
+            if (empty) v[j] = 0.0;
+            if (inf) v[j] = __longlong_as_double(0x7FF8000000000000LL);
+            const uint4 lcol = *reinterpret_cast<const uint4 *>(s_lc[c4 + j]);
+            const uint32_t both = (lrow.x & lcol.x) | (lrow.y & lcol.y) | (lrow.z & lcol.z) | (lrow.w & lcol.w);
+            if (both == 0 && abs(t3) < kSure && !empty && !inf && orow < nr && c4 + j < nc) {
+              v[j] = 0.0;
+              todo |= 1u << (j + (c4 >> 4) * 4);
+            }
           }
           // sums of earlier groups, behind a real branch: a predicated-off FP64
           // addition holds the FP64 unit like a full one
@@ -543,6 +613,9 @@ gemm_split_kernel(const SplitArgs g) {
 #pragma unroll
           for (int j = 0; j < 4; ++j) o[j] = v[j];
         }
+        if (__any_sync(0xffffffffu, todo != 0))
+          fallback(todo, Rp + s_roff[orow] + kgrp * g.R.s_k, g.R.s_k, Cp + kgrp * g.C.s_k, s_coff, g.C.s_k,
+                   min(k0, kend) - kgrp, tile + orow * Sm::kLdT, 4 * (warp >> 2));
         first = false;
         grp = 0;
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -557,6 +630,7 @@ gemm_split_kernel(const SplitArgs g) {
     if (grp == 0) {
       if (tid < kRows) s_er[tid] = s_mr[par][tid] + margin;
       else if (tid < kRows + NT) s_ec[tid - kRows] = s_mc[par][tid - kRows] + margin;
+      kgrp = k0;
       conv_sync();
     }
 #pragma unroll
@@ -570,6 +644,11 @@ gemm_split_kernel(const SplitArgs g) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) d[j] = digits(x[j], u == 2 ? base - (sh[j] >> 20) : base + (sh[j] >> 20));
       const int i = u == 2 ? ucol : urow;
+      // the other half of these eight k is with lane ^ 8
+      uint32_t big = large_bits(d) << (k & 4);
+      big |= __shfl_xor_sync(0xffffffffu, big, 8);
+      if (uh == 0)
+        reinterpret_cast<unsigned char *>(u == 2 ? s_lc[ucol] : s_lr[urow])[4 * grp + (k >> 3)] = (unsigned char)big;
       store_digits(d, x, sm + (u == 2 ? kABytes : 0) + ((i >> 3) * (kKc / 8) + (k >> 3)) * 128 + (i & 7) * 16 +
                              2 * (k & 4), (u == 2 ? NT : kRows) * kKc * 2);
     }
