@@ -47,7 +47,8 @@
 //      worse than a chain's bound, whatever the operands' grading.
 //      Outputs summed twice: none of Gaussian factors, 0.1% where entries are
 //      products of two or three Gaussians.
-// A row or column with a non-finite entry gives NaN in all its outputs.
+// Rows and columns with a non-finite entry go the same way, so infinities and NaN
+// come out where FP64 arithmetic puts them.
 //
 // Bound: issue slots of the conversion (about 40 instructions per operand
 // entry) and of the level combination (about 60 per output and group); FP64
@@ -592,12 +593,14 @@ gemm_split_kernel(const SplitArgs g) {
             const int ecj = s_ec[c4 + j];
             int32_t t3;
             v[j] = combine(L[j], eri + ecj, t3);
-            const bool empty = min(eri, ecj) < kEmpty / 2, inf = max(eri, ecj) > kNonfinite / 2;
+            // a row or column of zeros against finite entries: an exact zero. One with a
+            // non-finite entry has no digits and so no large bits
+            const bool inf = max(eri, ecj) > kNonfinite / 2;
+            const bool empty = min(eri, ecj) < kEmpty / 2 && !inf;
             if (empty) v[j] = 0.0;
-            if (inf) v[j] = __longlong_as_double(0x7FF8000000000000LL);
             const uint4 lcol = *reinterpret_cast<const uint4 *>(s_lc[c4 + j]);
             const uint32_t both = (lrow.x & lcol.x) | (lrow.y & lcol.y) | (lrow.z & lcol.z) | (lrow.w & lcol.w);
-            if (both == 0 && abs(t3) < kSure && !empty && !inf && orow < nr && c4 + j < nc) {
+            if (both == 0 && (abs(t3) < kSure || inf) && !empty && orow < nr && c4 + j < nc) {
               v[j] = 0.0;
               todo |= 1u << (j + (c4 >> 4) * 4);
             }

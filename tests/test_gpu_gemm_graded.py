@@ -121,3 +121,29 @@ def test_a_tensor_minus_its_orthogonal_form_is_zero(B, d, r):
     torch.cuda.synchronize()
     R = rnd.result()
     assert float(B.tt_dot(R, R)) <= 1e-24 * norm2
+
+
+@pytest.mark.parametrize("nb, M, N, K", [(3, 300, 90, 96), (1, 1031, 17, 250), (1, 4099, 330, 270)])
+def test_infinities_stay_infinities(B, nb, M, N, K):
+    """Infinities and NaN of an operand reach the outputs that FP64 arithmetic gives them, with
+    their sign, and no others."""
+    rng = np.random.default_rng(K)
+    A, Bm = rng.standard_normal((nb, M, K)), rng.standard_normal((nb, K, N))
+    A[0, 3, 1], A[-1, 7, K - 1], A[0, M - 1, K // 2] = np.inf, -np.inf, np.nan
+    A[0, 12, 5], A[0, 12, 40] = np.inf, -np.inf
+    Bm[0, 9, 2], Bm[-1, K - 3, N - 1] = -np.inf, np.inf
+    Bm[0, 1, 5] = 0.0                                       # 0 inf
+    C = B.gemm(torch.from_numpy(A).cuda(), torch.from_numpy(Bm).cuda())
+    torch.cuda.synchronize()
+    C = C.cpu().numpy()
+    rows = sorted({3, 7, M - 1, 12} | set(range(0, M, max(1, M // 40))))
+    A, C = A[:, rows], C[:, rows]
+    with np.errstate(invalid="ignore"):
+        ref = np.array([[[np.sum(a * b) for b in Bm[q].T] for a in A[q]] for q in range(nb)])
+        scale = np.array([[[np.sum(np.abs(a * b)) for b in Bm[q].T] for a in A[q]] for q in range(nb)])
+    assert np.isinf(ref).any() and np.isnan(ref).any()
+    assert np.array_equal(np.isnan(C), np.isnan(ref))
+    assert np.array_equal(C[np.isinf(ref)], ref[np.isinf(ref)])
+    fine = np.isfinite(ref)
+    u = 2.0 ** -53
+    assert np.all(np.abs(C - ref)[fine] <= 4 * K * u * scale[fine])
