@@ -321,10 +321,11 @@ int64_t tt_launch_count(void);
  * run: clears the control words and enqueues the persistent launch on
  *   `stream` and the larger pairs on the plan's streams, forked from and joined
  *   to `stream` (no synchronization; capturable once bound). spin_cap bounds each
- *   wait (polls of ~0.25 us; once any wait has run out every later wait gives
- *   up at once and the results are invalid).
+ *   wait of the persistent launch (polls of ~0.25 us; once any wait has run out every
+ *   later wait gives up at once and the results are invalid); a product of a pair on a
+ *   stream waits for the tensor cores up to a fixed limit (a second or so).
  * status: reads the status word of the last run (synchronizes `stream`):
- *   TT_OK, TT_ERR_TIMEOUT if a wait ran out, TT_ERR_NONFINITE if a norm or a
+ *   TT_OK, TT_ERR_TIMEOUT if a wait ran out in either form, TT_ERR_NONFINITE if a norm or a
  *   Gram matrix was not finite (NaN or Inf in an input), TT_ERR_BREAKDOWN.
  * info: number of stages and tasks of the bound plan's engine launch (0 when
  *   every pair runs on a stream) and its resident CTAs.

@@ -169,7 +169,11 @@ cudaError_t clear_device_error();
 // bit owns its word; read_device_error ORs them.
 constexpr int kHealthTimeout = 1, kHealthNonfinite = 2, kHealthBreakdown = 4;
 cudaError_t qr_health_word(int *value, bool clear);
-// Where the calling thread's next factorizations and norms note their bits: a
+// Polls of one wait for tensor-core products before it gives up (the kernel then sets
+// kHealthTimeout and writes NaN), and the limit in force.
+constexpr long long kMmaWaits = 2000000;
+long long mma_waits();
+// Where the calling thread's next products, factorizations and norms note their bits: a
 // device word of the caller (a batched plan's status), or nullptr for the
 // device error word.
 void set_health_word(int *word);

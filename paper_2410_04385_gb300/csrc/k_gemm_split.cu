@@ -85,7 +85,6 @@ constexpr int kABytes = kDig * kRows * kKc * 2;
 constexpr int kNonfinite = 1 << 20;      // row / column exponent of a non-finite entry
 constexpr int kEmpty = -(1 << 20);       // exponent of an all-zero row / column
 constexpr int kSure = 5200;              // 2^20 2^-7.66: a sum this large is no cancelled one
-constexpr long long kSplitWaitLimit = 2000000;
 
 // Shared memory of the NT-column form: digits of both operands, raw tiles,
 // output tile (FP64). More than half an SM's, so one CTA per SM, whose
@@ -137,6 +136,8 @@ struct SplitArgs {
   const double *alpha_dev;
   const int *skip_dev;
   double *partial;
+  int *health;                           // where a wait that ran out is noted: the caller's word or null
+  long long waits;                       // polls of one wait
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
@@ -548,10 +549,19 @@ gemm_split_kernel(const SplitArgs g) {
     if (grp > 0) {
       // the digit products issued last (bounded wait)
       uint32_t done = 0;
-      for (long long w = 0; w < kSplitWaitLimit && !done; ++w)
+      for (long long w = 0; w < g.waits && !done; ++w)
         asm volatile("{\n.reg .pred pr;\nmbarrier.try_wait.parity.shared::cta.b64 pr, [%1], %2;\n"
                      "selp.u32 %0, 1, 0, pr;\n}\n"
                      : "=r"(done) : "r"(smem_u32(&s_bar)), "r"(phase) : "memory");
+      // after giving up: the products still read shared and write tensor memory, so
+      // they get another (bounded) wait before either goes
+      for (long long w = 0, late = done; w < kMmaWaits && !late; ++w) {
+        uint32_t p;
+        asm volatile("{\n.reg .pred pr;\nmbarrier.try_wait.parity.shared::cta.b64 pr, [%1], %2;\n"
+                     "selp.u32 %0, 1, 0, pr;\n}\n"
+                     : "=r"(p) : "r"(smem_u32(&s_bar)), "r"(phase) : "memory");
+        late = p;
+      }
       phase ^= 1u;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       // a group ends when it is full, or an entry exceeds its row's or
@@ -670,7 +680,7 @@ gemm_split_kernel(const SplitArgs g) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(s_taddr), "r"(Sm::kTmem)
                  : "memory");
   if (fail) {
-    if (tid == 0) atomicExch(&g_split_error, 1);
+    if (tid == 0) atomicOr(g.health != nullptr ? g.health : &g_split_error, kHealthTimeout);
     for (int e = tid; e < kRows * NT; e += kThreadsS)
       tile[(e / NT) * Sm::kLdT + e % NT] = __longlong_as_double(0x7FF8000000000000LL);
     __syncthreads();
@@ -828,6 +838,8 @@ SplitPlan orient(const Gemm &q, bool swap, int nt) {
   g.alpha_dev = q.alpha_dev;
   g.skip_dev = q.skip_dev;
   g.partial = nullptr;
+  g.health = nullptr;
+  g.waits = kMmaWaits;
   L.batch = batch;
   return L;
 }
@@ -951,6 +963,8 @@ cudaError_t gemm_split(const Gemm &q, double *scratch, cudaStream_t st) {
   if (L.g.ksplit > 1 && scratch == nullptr) return cudaErrorInvalidValue;
   if (L.blocks >= (1LL << 31)) return cudaErrorInvalidConfiguration;
   L.g.partial = scratch;
+  L.g.health = health_target();
+  L.g.waits = mma_waits();
   const cudaError_t e = L.nt == 64 ? launch_split<64>(L, st) : L.nt == 48 ? launch_split<48>(L, st)
                                                                           : launch_split<32>(L, st);
   if (e != cudaSuccess || L.g.ksplit == 1) return e;

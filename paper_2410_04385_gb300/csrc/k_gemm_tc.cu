@@ -24,6 +24,7 @@
 // always fit in the 512 columns of an SM and tcgen05.alloc never waits.
 #include <algorithm>
 #include <cstdint>
+#include <cstdlib>
 #include "hatt_internal.cuh"
 
 namespace hatt {
@@ -37,7 +38,6 @@ constexpr int kTcM = 128;
 constexpr int kTcMaxN = 256;
 constexpr int kSliceBytes = 128;                 // K bytes per staged slice and row
 constexpr int kTcSmem = 100 * 1024;              // caps residency at 2 blocks per SM
-constexpr long long kWaitLimit = 2000000;        // mbarrier polls before giving up
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
   return (uint32_t)__cvta_generic_to_shared(p);
@@ -93,7 +93,7 @@ __device__ __forceinline__ void stage(const Operand &op, int r0, int nrows, int 
 template <bool TF32>
 __global__ void __launch_bounds__(kTcThreads)
 gemm_tc_kernel(Gemm g, int swap, int bn, int tiles_n, int tiles_m, int ksplit, int kchunk,
-               int tmem_cols, double *partial, int *counters) {
+               int tmem_cols, double *partial, int *counters, int *health, long long waits) {
   pdl_enter();
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ uint32_t s_taddr;
@@ -173,18 +173,24 @@ gemm_tc_kernel(Gemm g, int swap, int bn, int tiles_n, int tiles_m, int ksplit, i
     }
     any = true;
     uint32_t done = 0;
-    for (long long it = 0; it < kWaitLimit && !done; ++it)
+    for (long long it = 0; it < waits && !done; ++it)
+      asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+                   "selp.u32 %0, 1, 0, p;\n}\n"
+                   : "=r"(done) : "r"(smem_u32(&s_bar)), "r"(phase) : "memory");
+    if (!done) s_fail = 1;
+    // after giving up: the products still read shared and write tensor memory, so
+    // they get another (bounded) wait before either goes
+    for (long long it = 0; it < kMmaWaits && !done; ++it)
       asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
                    "selp.u32 %0, 1, 0, p;\n}\n"
                    : "=r"(done) : "r"(smem_u32(&s_bar)), "r"(phase) : "memory");
     phase ^= 1u;
-    if (!done) s_fail = 1;
     __syncthreads();
     if (s_fail) break;
   }
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const bool fail = s_fail != 0;
-  if (fail && tid == 0) atomicExch(&g_device_error, 1);
+  if (fail && tid == 0) atomicOr(health != nullptr ? health : &g_device_error, kHealthTimeout);
 
   // epilogue: thread = tile row (lane quarter of its warp), columns in 8s
   const double alpha = g.alpha * (g.alpha_dev ? *g.alpha_dev : 1.0);
@@ -275,6 +281,16 @@ TcLaunch tc_plan(const Gemm &g) {
 
 }  // namespace
 
+// HATT_MMA_WAITS=<n> (read once), a test hook: a wait for tensor-core products gives
+// up after n polls (0: at once), so that the timeout status comes without a hang.
+long long mma_waits() {
+  static const long long v = [] {
+    const char *e = getenv("HATT_MMA_WAITS");
+    return e != nullptr && *e != 0 ? std::max(0LL, (long long)atoll(e)) : kMmaWaits;
+  }();
+  return v;
+}
+
 cudaError_t read_device_error(int *value) {
   int split = 0, qr = 0, misc = 0, refine = 0;
   cudaError_t e = cudaMemcpyFromSymbol(value, g_device_error, sizeof(int));
@@ -317,12 +333,14 @@ cudaError_t gemm_tc(const Gemm &g, double *scratch, int *counters, cudaStream_t 
     e = cudaFuncSetAttribute(gemm_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
     if (e != cudaSuccess) return e;
     launch_k(gemm_tc_kernel<true>, (unsigned)blocks, kTcThreads, kTcSmem, st, 
-        g, L.swap, L.bn, L.tiles_n, L.tiles_m, L.ksplit, L.kchunk, L.tmem_cols, scratch, counters);
+        g, L.swap, L.bn, L.tiles_n, L.tiles_m, L.ksplit, L.kchunk, L.tmem_cols, scratch, counters,
+        health_target(), mma_waits());
   } else {
     e = cudaFuncSetAttribute(gemm_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
     if (e != cudaSuccess) return e;
     launch_k(gemm_tc_kernel<false>, (unsigned)blocks, kTcThreads, kTcSmem, st, 
-        g, L.swap, L.bn, L.tiles_n, L.tiles_m, L.ksplit, L.kchunk, L.tmem_cols, scratch, counters);
+        g, L.swap, L.bn, L.tiles_n, L.tiles_m, L.ksplit, L.kchunk, L.tmem_cols, scratch, counters,
+        health_target(), mma_waits());
   }
   note_launch();
   return cudaGetLastError();

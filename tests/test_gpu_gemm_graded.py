@@ -146,4 +146,4 @@ def test_infinities_stay_infinities(B, nb, M, N, K):
     assert np.array_equal(C[np.isinf(ref)], ref[np.isinf(ref)])
     fine = np.isfinite(ref)
     u = 2.0 ** -53
-    assert np.all(np.abs(C - ref)[fine] <= 4 * K * u * scale[fine])
+    assert np.all(np.abs(C[fine] - ref[fine]) <= 4 * K * u * scale[fine])
