@@ -303,8 +303,8 @@ oa_cluster_kernel(const double *G, int c, double *Uout, double floor_norm, const
   double *Gs = sm;                     // c x c
   double *Us = Gs + c * c;             // c x c
   double *lam = Us + c * c;            // c
-  double *part = lam + c;              // 3 x kMaxCluster
-  double *work = part + 3 * kMaxCluster;
+  double *part = lam + c;              // 4 x kMaxCluster
+  double *work = part + 4 * kMaxCluster;
   double *Rs = work, *Ts = Rs + c * w, *Ss = Ts + c * w, *Ns = Ss + c * w;
   __shared__ double red[33];
   __shared__ double s_gn, s_delta, s_inv, s_stop;
@@ -322,6 +322,11 @@ oa_cluster_kernel(const double *G, int c, double *Uout, double floor_norm, const
   const double u = 1.1102230246251565e-16;
   for (int it = 0; it < kRefine + kOrth; ++it) {
     const bool orth = it >= kRefine;
+    // the CTAs' largest corrections: a closing step writes them before its first
+    // barrier, while a slower CTA may still read those of the step before, so two
+    // buffers (one value read twice would let the CTAs stop at different steps, with
+    // writes to the shared memory of a CTA that has left)
+    const int largest = (2 + (it & 1)) * kMaxCluster;
     // R = I - U^T U and T = G U on the own columns, then S = U^T T
     for (int e = tid; e < c * wl; e += nt) {
       const int i = e / wl, jj = e - i * wl, j = j0 + jj;
@@ -408,7 +413,7 @@ oa_cluster_kernel(const double *G, int c, double *Uout, double floor_norm, const
     }
     emax = blk_reduce(emax, red, true);
     if (tid == 0)
-      for (int q = 0; q < P; ++q) cl.map_shared_rank(part, q)[2 * kMaxCluster + rank] = emax;
+      for (int q = 0; q < P; ++q) cl.map_shared_rank(part, q)[largest + rank] = emax;
     cl.sync();                         // every CTA has finished reading U
     for (int q = 0; q < P; ++q) {
       double *dst = cl.map_shared_rank(Us, q);
@@ -420,7 +425,7 @@ oa_cluster_kernel(const double *G, int c, double *Uout, double floor_norm, const
     cl.sync();
     if (tid == 0) {
       double mx = 0.0;
-      for (int q = 0; q < P; ++q) mx = fmax(mx, part[2 * kMaxCluster + q]);
+      for (int q = 0; q < P; ++q) mx = fmax(mx, part[largest + q]);
       s_stop = (mx <= kStepConverged) ? 1.0 : 0.0;
     }
     __syncthreads();
@@ -436,7 +441,7 @@ int cluster_size_for(int c) { return c >= 32 ? 16 : (c >= 8 ? 8 : 1); }
 
 size_t refine_smem(int c, int P) {
   const int w = (c + P - 1) / P;
-  return ((size_t)2 * c * c + c + 3 * kMaxCluster + (size_t)4 * c * w) * sizeof(double);
+  return ((size_t)2 * c * c + c + 4 * kMaxCluster + (size_t)4 * c * w) * sizeof(double);
 }
 
 size_t columns_smem(int c, int blocks) {
