@@ -320,10 +320,15 @@ int64_t tt_launch_count(void);
  *   `stream`; not allowed while it is being captured.
  * run: clears the control words and enqueues the persistent launch on
  *   `stream` and the larger pairs on the plan's streams, forked from and joined
- *   to `stream` (no synchronization; capturable once bound). spin_cap bounds each
- *   wait of the persistent launch (polls of ~0.25 us; once any wait has run out every
- *   later wait gives up at once and the results are invalid); a product of a pair on a
- *   stream waits for the tensor cores up to a fixed limit (a second or so).
+ *   to `stream` (no synchronization; capturable once bound). The persistent
+ *   launch is one launch; the pairs on streams are issued by the calling thread, about
+ *   57 us of launches per core (3.5 s for 256 uneven pairs of order 10 to 20 and ranks
+ *   8 to 40: the call returns when nearly all of its work is done). A caller that
+ *   needs its thread meanwhile captures the run once and launches the graph.
+ *   spin_cap bounds each wait of the persistent launch (polls of ~0.25 us; once any
+ *   wait has run out every later wait gives up at once and the results are invalid); a
+ *   product of a pair on a stream waits for the tensor cores up to a fixed limit (a
+ *   second or so).
  * status: reads the status word of the last run (synchronizes `stream`):
  *   TT_OK, TT_ERR_TIMEOUT if a wait ran out in either form, TT_ERR_NONFINITE if a norm or a
  *   Gram matrix was not finite (NaN or Inf in an input), TT_ERR_BREAKDOWN.

@@ -614,7 +614,9 @@ class BatchedRecompressor:
     """Many independent pairs recompressed in one call (tt_batched_*): the small
     ones by one persistent launch of the task engine, the larger ones on streams
     that the plan owns. Plans once, owns every output buffer and the workspace;
-    `run` enqueues the work (capturable after construction)."""
+    `run` enqueues the work (capturable after construction). The larger pairs are
+    issued launch by launch from the calling thread, about 57 us per core; capture
+    the run in a CUDA graph where that thread has other work."""
 
     def __init__(self, pairs, autotune: bool = True, stream=None):
         """pairs: list of (Y cores, Z cores, options dict) with CUDA float64
