@@ -37,21 +37,32 @@ SKETCH_SEED = 9
 L2_FLUSH_BYTES = 256 << 20          # > 129 MB L2
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12   # SMs x FP64 FMA lanes/SM x 2 x max clock
 FP64_PEAK_NOTE = ("derived: 152 SMs x 2 FP64 FMA lanes/SM/clk x 2 flop x 2070 MHz = 1.259 TFLOP/s; "
-                  "a DFMA throughput loop measured 1.196 TFLOP/s; most of these products run on the "
-                  "tensor cores from exact 8-bit digits, so a fraction may exceed 1")
+                  "a DFMA throughput loop measured 1.196 TFLOP/s")
+
+
+def digit_peak():
+    """(FP64 TFLOP/s the tensor cores allow, where it comes from): an FP64 product is 36 digit
+    products at the 16-bit rate measured on this card."""
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
+            rate, src = float(json.load(f)["bf16_tflops"]), "measured"
+    except (OSError, ValueError, KeyError):
+        rate, src = 1900.0, "an earlier measurement"
+    return rate / 36.0, (f"{src} 16-bit tensor rate {rate:.0f} TFLOP/s / 36 digit products per FP64 product; "
+                         f"the FP64 pipe's peak is {FP64_PEAK_TFLOPS:.3f} TFLOP/s ({FP64_PEAK_NOTE})")
 
 
 GEMM_TIMING_STEPS = 3
 CFG3_GOLDEN = os.path.join(ROOT, "tests", "golden", "cfg3_oracle_samples.npz")
 AC_GOLDEN = os.path.join(ROOT, "tests", "golden", "allen_cahn_oracle_samples.npz")
 GEMM_PROFILE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "profiles",
-                            "gemm_f64_kernel_d20_traffic.json")
+                            "gemm_split_kernel_d20_traffic.json")
 GEMM_SOURCE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "paper_2410_04385_gb300",
-                           "csrc", "k_gemm.cu")
+                           "csrc", "k_gemm_split.cu")
 
 
 def gemm_traffic_per_launch():
-    """(DRAM bytes read + written per launch of the method GEMMs, note) from
+    """(DRAM bytes read + written per launch of the method's digit products, note) from
     the committed ncu summary. The bytes are None when the kernel source has
     changed since the capture, and the note says so."""
     try:
@@ -62,7 +73,7 @@ def gemm_traffic_per_launch():
     except (OSError, ValueError) as e:
         return None, f"no ncu record ({type(e).__name__})"
     if prof.get("source_sha256") != sha:
-        return None, "stale: k_gemm.cu changed since the ncu capture; re-capture"
+        return None, "stale: k_gemm_split.cu changed since the ncu capture; re-capture"
     return prof.get("dram_bytes_per_launch"), prof.get("note", "ncu capture")
 
 
@@ -301,8 +312,9 @@ def run_batch_cfg4(binding, workloads, dev, rank=0, world=1):
         n, r, s_, ell = sharding.pair_ranks(Y, Z, o)
         sw += costmodel.hatt1_flops(n, r, s_, ell)[1]
     ach = sw / (min(ms) * 1e-3) / 1e12
-    out["engine_roofline"] = {"bound": "alu", "fp64_flops": sw, "achieved": ach, "peak": FP64_PEAK_TFLOPS,
-                              "unit": "TFLOP/s", "frac": ach / FP64_PEAK_TFLOPS,
+    peak, _ = digit_peak()
+    out["engine_roofline"] = {"bound": "alu", "fp64_flops": sw, "achieved": ach, "peak": peak,
+                              "unit": "TFLOP/s", "frac": ach / peak, "of_fp64_pipe": ach / FP64_PEAK_TFLOPS,
                               "note": "FP64 left-to-right pass (Section 4 model) over the batch time; the "
                                       "FP32 sketch products (HPCRL) run inside the same time"}
     out["device_error"] = binding.device_error()
@@ -733,6 +745,7 @@ def main():
     aux_ms = sum(g_ms[i] for i in a_idx)
     meth_tflops = meth_flops / (meth_ms * 1e-3) / 1e12
     traffic, traffic_note = gemm_traffic_per_launch()
+    peak, peak_note = digit_peak()
 
     # ---- roofline of the whole step (one graph launch = one recompression) ----
     n = workloads.modes_of(Y)
@@ -760,8 +773,9 @@ def main():
         "roofline": {"bound": "alu",
                      "kernel": "FP64 products (digits on tcgen05, small, DFMA tiles), launches computing the HaTT contractions (HPCRL S1-S3, "
                                "C_k W, Q^T C_k, the two core-update stages)",
-                     "achieved": meth_tflops, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                     "frac": meth_tflops / FP64_PEAK_TFLOPS, "traffic": traffic,
+                     "achieved": meth_tflops, "peak": peak, "unit": "TFLOP/s",
+                     "frac": meth_tflops / peak, "of_fp64_pipe": meth_tflops / FP64_PEAK_TFLOPS,
+                     "traffic": traffic,
                      "traffic_note": traffic_note,
                      "launches_timed": len(m_idx),
                      "avg_launch_us": 1e3 * meth_ms / max(len(m_idx), 1),
@@ -771,7 +785,7 @@ def main():
                      "share_of_step": meth_ms / timed_steps_ms,
                      "timing": "CUDA events around every launch on its own stream (library kernel "
                                "timer), eager steps queued behind a GPU sleep",
-                     "peak_source": FP64_PEAK_NOTE},
+                     "peak_source": peak_note},
         "gemm_aux": {"kernel": "FP64 products, all other launches (truncation Gram matrices and "
                                "projections; the Cholesky QR computes its Gram matrix in its own "
                                "kernel)",
@@ -779,8 +793,8 @@ def main():
                      "share_of_step": aux_ms / timed_steps_ms,
                      "all_gemm_share_of_step": gemm_ms / timed_steps_ms},
         "roofline_step": {"bound": "alu", "kernel": "HaTT-1 step (graph of all libhatt kernels)",
-                          "achieved": achieved_tflops, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                          "frac": achieved_tflops / FP64_PEAK_TFLOPS,
+                          "achieved": achieved_tflops, "peak": peak, "unit": "TFLOP/s",
+                          "frac": achieved_tflops / peak, "of_fp64_pipe": achieved_tflops / FP64_PEAK_TFLOPS,
                           "algorithmic_flops_per_step": alg_flops},
         "clocks": clocks,
     }

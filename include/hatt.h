@@ -322,8 +322,8 @@ int64_t tt_launch_count(void);
  *   `stream` and the larger pairs on the plan's streams, forked from and joined
  *   to `stream` (no synchronization; capturable once bound). The persistent
  *   launch is one launch; the pairs on streams are issued by the calling thread, about
- *   57 us of launches per core (3.5 s for 256 uneven pairs of order 10 to 20 and ranks
- *   8 to 40: the call returns when nearly all of its work is done). A caller that
+ *   57 us of launches per core (3.5 s for 256 uneven pairs of order 10 to 40 and ranks
+ *   8 to 48: the call returns when nearly all of its work is done). A caller that
  *   needs its thread meanwhile captures the run once and launches the graph.
  *   spin_cap bounds each wait of the persistent launch (polls of ~0.25 us; once any
  *   wait has run out every later wait gives up at once and the results are invalid); a

@@ -50,11 +50,18 @@
 // Rows and columns with a non-finite entry go the same way, so infinities and NaN
 // come out where FP64 arithmetic puts them.
 //
-// Bound: issue slots of the conversion (about 40 instructions per operand
-// entry) and of the level combination (about 60 per output and group); FP64
-// instructions appear only in the sums over groups and in alpha. 512 threads,
-// one CTA per SM: with NT = 64 an entry of the row operand is converted once
-// per 64 columns, which two CTAs of 32 columns each would do twice. Outputs
+// Bound: ALU instructions of the conversion (about 45 per operand entry) and of the
+// level combination (about 65 per output and group), behind barriers: one digit
+// buffer, so conversion and tensor work take turns. ncu at 5760 x 90 x 1600 (NT = 48,
+// 450 blocks, 202 us): ALU pipe 54% of active cycles, issue slots 49%, tensor pipe
+// 14%, DRAM 5% (79 MB, each operand once); warps wait for barriers, shared memory and
+// dependent instructions in equal parts. FP64 instructions appear only in the sums
+// over groups, in alpha and in step 7. Step 7's test costs 3 to 5% (12 cores of modes
+// 64, ranks 40 x 40, sketch 90: 24.2 -> 25.1 ms); operands that need the FP64 sums
+// cost more: at 5760 x 90 x 1600 210 us for Gaussian ones, 520 for blocks 2^60 apart,
+// 3450 where every entry has a size of its own (DFMA tiles: 1480 for all).
+// 512 threads, one CTA per SM: with NT = 64 an entry of the row operand is converted
+// once per 64 columns, which two CTAs of 32 columns each would do twice. Outputs
 // are combined in a loop over four columns (1700 to 2400 clocks each: 64-bit
 // integer multiply-adds, leading-zero counts and one FP64 add run at a quarter
 // of the issue rate and less); unrolled over 16 the code is 100 KB and no faster.
