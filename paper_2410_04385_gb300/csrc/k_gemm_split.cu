@@ -885,7 +885,7 @@ void plan_split(SplitPlan &L) {
 // the DFMA product is predicted at 230 multiply-adds per clock (75% of the FP64
 // units, what its mid-sized products reach) plus 12000 clocks. Measured on both
 // sides of the line (us, digits against DFMA): 1 x 50 x 50 x 1600 20 and 24,
-// 400 x 100 x 100 13 and 20, 50 x 1600 x 50 15 and 13, 200 x 100 x 100 13 and 12.
+// 400 x 100 x 100 14 and 20, 50 x 1600 x 50 15 and 13, 300 x 100 x 100 14 and 10.
 Choice choose(const Gemm &q) {
   using Key = std::array<int, 6>;
   struct Hash {
